@@ -246,7 +246,11 @@ int dpdr_plan_set(dpdr_plan_t plan, int key, int64_t value);
  *   [17] CTA layout of the schedule kernels: 1 rank ranges, 2 by work
  *        (DPDR_OPT_SCHED_LAYOUT; flagged words always take rank ranges)
  *   [18] block passes of the counters transport: 1 per-lane copies, 2 bulk
- *        copies (DPDR_OPT_SCHED_COPY) */
+ *        copies (DPDR_OPT_SCHED_COPY)
+ *   [19] subtree cells of the schedule kernels, 0 when they do not run on
+ *        cells.  They do while every schedule option is automatic and one
+ *        column slice of the cells fits the GPU at once; [5], [6], [12],
+ *        [17] and [18] then describe the layout that they replace */
 int dpdr_plan_info(dpdr_plan_t plan, int64_t* info, int n);
 
 /* Releases the plan's device and host memory.  The caller must first make

@@ -145,7 +145,7 @@ INFO_KEYS = ("p", "m", "b", "max_depth", "auto_mode", "sched_ctas",
              "sched_ranks_per_cta", "scratch_bytes", "vector_path",
              "split_depth", "split_subtrees", "split_group", "sched_slices",
              "topology", "host_path", "sched_transport", "tree_width",
-             "sched_layout", "sched_copy")
+             "sched_layout", "sched_copy", "sched_cells")
 
 
 class Plan:

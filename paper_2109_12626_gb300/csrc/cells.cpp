@@ -1,0 +1,251 @@
+// cells.cpp -- host side of the schedule kernels on subtree cells: how the
+// trees are cut into cells, the cells' device descriptors, their column
+// slices, scratch and launches (schedule_cells.cuh, schedule_words.cu).
+#include <algorithm>
+#include <cstring>
+#include <map>
+
+#include "dpdr_internal.h"
+
+namespace dpdr {
+namespace {
+
+// One way to cut a subtree: its open piece (the part that holds the subtree's
+// root) joins what lies above, the cells below it are closed.
+struct Cut {
+    int tiers, cells;   // cells on the longest path below the piece; cells below
+    bool join;          // the node's children are in its piece, as pieces s0, s1
+    int s0, s1;
+    bool operator<(const Cut& o) const { return tiers != o.tiers ? tiers < o.tiers : cells < o.cells; }
+};
+constexpr int kNoCut = 1 << 28;
+
+struct HostCell {
+    std::vector<int> ranks;  // post-order, the cell's root last
+    int root, depth, par_cell, par_rank, nlev;
+};
+
+// The cells of the plan's trees.  A node's children are both in its cell or
+// both roots of other cells, and a cell holds at most max_ranks ranks on
+// max_levels levels.  Of all such cuts: the fewest cells between a leaf and
+// the root (each costs an exchange through L2 each way), then the fewest
+// cells.  Subtrees of a complete tree that have the same size have the same
+// shape, so the best cut is found once per size; pieces are numbered
+// (ranks - 1) * max_levels + (levels - 1).
+void cut_cells(const Plan* P, int max_ranks, int max_levels, std::vector<HostCell>* cells,
+               std::vector<int>* cell_of, std::vector<char>* top_of)
+{
+    const int p = P->p, pieces = max_ranks * max_levels;
+    std::vector<int> size(p), piece(p, 0);
+    std::vector<int>& cell = *cell_of;
+    std::vector<char>& top = *top_of;
+    cell.assign(p, -1);
+    top.assign(p, 0);
+    std::map<int, std::vector<Cut>> cuts;
+    auto best = [](const std::vector<Cut>& c) { return int(std::min_element(c.begin(), c.end()) - c.begin()); };
+    for (int i = 0; i < p; i++) {  // post-order: children first
+        const int c0 = P->child0[i], c1 = P->child1[i];
+        size[i] = 1 + (c0 >= 0 ? size[c0] : 0) + (c1 >= 0 ? size[c1] : 0);
+        std::vector<Cut>& c = cuts[size[i]];
+        if (!c.empty()) continue;
+        c.assign(pieces, Cut{kNoCut, 0, false, 0, 0});
+        if (c0 < 0) {
+            c[0] = Cut{0, 0, false, 0, 0};
+            continue;
+        }
+        const std::vector<Cut>& a = cuts[size[c0]];
+        const std::vector<Cut>& d = c1 >= 0 ? cuts[size[c1]] : a;
+        if (c1 >= 0) {
+            const Cut x = a[best(a)], y = d[best(d)];
+            c[0] = Cut{1 + std::max(x.tiers, y.tiers), 2 + x.cells + y.cells, false, 0, 0};
+        }
+        for (int s0 = 0; s0 < pieces; s0++) {
+            if (a[s0].tiers >= kNoCut) continue;
+            for (int s1 = 0; s1 < (c1 >= 0 ? pieces : 1); s1++) {
+                const Cut x = a[s0], y = c1 >= 0 ? d[s1] : Cut{0, 0, false, 0, 0};
+                if (y.tiers >= kNoCut) continue;
+                const int n = 1 + s0 / max_levels + 1 + (c1 >= 0 ? s1 / max_levels + 1 : 0);
+                const int l = 1 + std::max(s0 % max_levels + 1, c1 >= 0 ? s1 % max_levels + 1 : 0);
+                if (n > max_ranks || l > max_levels) continue;
+                Cut& b = c[(n - 1) * max_levels + l - 1];
+                const Cut j{std::max(x.tiers, y.tiers), x.cells + y.cells, true, s0, s1};
+                if (j < b) b = j;
+            }
+        }
+    }
+    for (int i = p - 1; i >= 0; i--) {  // parents first: the pieces chosen
+        if (P->parent[i] < 0) top[i] = 1;
+        const std::vector<Cut>& c = cuts[size[i]];
+        if (top[i]) piece[i] = best(c);
+        const int c0 = P->child0[i], c1 = P->child1[i];
+        if (c0 < 0) continue;
+        const Cut& k = c[piece[i]];
+        top[c0] = !k.join;
+        piece[c0] = k.s0;
+        if (c1 >= 0) {
+            top[c1] = !k.join;
+            piece[c1] = k.s1;
+        }
+    }
+    cells->clear();
+    for (int i = 0; i < p; i++)
+        if (top[i]) {
+            cell[i] = int(cells->size());
+            cells->push_back(HostCell());
+        }
+    for (int i = p - 1; i >= 0; i--)
+        if (cell[i] < 0) cell[i] = cell[P->parent[i]];
+    for (int i = 0; i < p; i++) (*cells)[cell[i]].ranks.push_back(i);
+    for (HostCell& c : *cells) {
+        c.root = c.ranks.back();
+        c.depth = P->depth[c.root];
+        c.par_rank = P->parent[c.root];
+        c.par_cell = c.par_rank < 0 ? -1 : cell[c.par_rank];
+        c.nlev = 0;
+        for (int i : c.ranks) c.nlev = std::max(c.nlev, P->depth[i] - c.depth + 1);
+    }
+}
+
+bool is_second(const Plan* P, int i) { return P->parent[i] >= 0 && P->child1[P->parent[i]] == i; }
+
+}  // namespace
+
+void make_cells(const Plan* P, int max_ranks, int max_levels, CellPlan* C, std::vector<CellDesc>* out)
+{
+    std::vector<HostCell> cells;
+    std::vector<int> cell;
+    std::vector<char> top;
+    cut_cells(P, max_ranks, max_levels, &cells, &cell, &top);
+    out->assign(cells.size(), CellDesc());
+    C->n = int(cells.size());
+    C->root0 = P->r0 >= 0 ? cell[P->r0] : -1;
+    C->root1 = cell[P->r1];
+    C->down = C->ranks = 0;
+    for (size_t k = 0; k < cells.size(); k++) {
+        const HostCell& h = cells[k];
+        CellDesc& c = (*out)[k];
+        std::memset(&c, 0, sizeof c);
+        c.n = int(h.ranks.size());
+        C->ranks = std::max(C->ranks, c.n);
+        c.root = h.root;
+        c.depth = h.depth;
+        c.par_cell = h.par_cell;
+        c.par_rank = h.par_rank;
+        c.nlev = h.nlev;
+        unsigned again = h.nlev > 1 ? 1u << (c.n - 1) : 0u;  // positions whose finals are read again
+        for (int t = 0; t < c.n; t++) {
+            const int i = h.ranks[t], c0 = P->child0[i], c1 = P->child1[i];
+            const bool in = c0 >= 0 && !top[c0];
+            const int pos1 = in && c1 >= 0
+                ? int(std::find(h.ranks.begin(), h.ranks.end(), c1) - h.ranks.begin()) : 0;
+            c.rank[t] = i;
+            c.node_par[t] = i == h.root ? -1 : P->parent[i];
+            c.tape[t] = (in ? (c1 >= 0 ? 2 : 1) : 0) | (i != h.root && is_second(P, i) ? 4 : 0) |
+                        (pos1 << 3);
+            if (c0 >= 0 && !in) {  // two children: a single one always joins
+                c.ext_k[c.next] = t;
+                c.ext_cell[2 * c.next] = cell[c0];
+                c.ext_cell[2 * c.next + 1] = cell[c1];
+                c.ext_rank[2 * c.next] = c0;
+                c.ext_rank[2 * c.next + 1] = c1;
+                c.next++;
+                again |= 1u << t;
+            }
+        }
+        int t = 0;
+        for (int l = 0; l < kCellLevels; l++) {
+            c.lev_off[l] = t;
+            for (int q = 0; q < c.n; q++)
+                if (P->depth[h.ranks[q]] - h.depth == l) {
+                    if ((again >> q) & 1u) c.reread |= 1 << t;
+                    c.lev_k[t++] = q;
+                }
+        }
+        c.lev_off[kCellLevels] = t;
+        c.down = c.next ? C->down++ : 0;
+    }
+    for (CellDesc& c : *out) c.par_down = c.par_cell < 0 ? 0 : (*out)[c.par_cell].down;
+}
+
+// Slices of 32 units, as many side by side as there are warps for (but for a
+// slice of the row's last elements), in as few waves as that takes.
+CellSlices cell_slices(const Plan* P, const CellPlan& C, bool vec)
+{
+    const int64_t epu = vec ? 16 / int64_t(P->esize) : 1;
+    const int64_t maxblk = (P->m + P->b - 1) / P->b;
+    // bounds are rounded up to units, so a block may hold one more
+    const int64_t units = std::max<int64_t>(1, (maxblk + epu - 1) / epu + (epu > 1 && P->b > 1 ? 1 : 0));
+    const int64_t slices = (units + 31) / 32, cap = C.warps / C.n - cell_tail(P, vec);
+    const int64_t waves = (slices + cap - 1) / cap;
+    return CellSlices{int((slices + waves - 1) / waves), int(waves)};
+}
+
+// Whether a call on aligned buffers moves 16-byte units: not when blocks are
+// so short that rounding their bounds to units would change them by much.
+bool cell_vector(const Plan* P)
+{
+    return P->last_vector_path && (P->esize == 16 || P->m / P->b >= 64);
+}
+
+int cell_tail(const Plan* P, bool vec) { return vec && P->m % (16 / int64_t(P->esize)) ? 1 : 0; }
+
+// The cells' device memory: control words (epoch 1 first), descriptors at 256,
+// scratch (zeroed) at off_scratch.
+int cell_scratch(Plan* P, CellPlan* C, const void* desc, size_t desc_bytes)
+{
+    const size_t bytes = C->off_scratch + C->scratch;
+    cudaError_t e;
+    if (bytes > C->bytes) {
+        if (C->d) cudaFree(C->d);
+        C->d = nullptr;
+        C->bytes = 0;
+        e = cudaMalloc(&C->d, bytes);
+        if (e != cudaSuccess) {
+            C->d = nullptr;
+            return cuda_fail(e, "schedule cells: cudaMalloc");
+        }
+        C->bytes = bytes;
+    }
+    const uint32_t one = 1;
+    e = cudaMemset(C->d, 0, bytes);
+    if (e == cudaSuccess) e = cudaMemcpy(C->d, &one, sizeof one, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(C->d + 256, desc, desc_bytes, cudaMemcpyHostToDevice);
+    return e == cudaSuccess ? DPDR_OK : cuda_fail(e, "schedule cells: upload");
+}
+
+int cell_launch(const void* kernel, void* args, int64_t warps, int per_cta, size_t smem, cudaStream_t s)
+{
+    void* argv[] = {args};
+    const cudaError_t e = cudaLaunchCooperativeKernel(
+        kernel, dim3(unsigned((warps + per_cta - 1) / per_cta)), dim3(unsigned(32 * per_cta)), argv, smem, s);
+    if (e == cudaErrorCooperativeLaunchTooLarge) {
+        cudaGetLastError();
+        return fail(DPDR_ERR_NOT_COOPERATIVE, "schedule kernel: CTAs cannot be co-resident");
+    }
+    return e == cudaSuccess ? DPDR_OK : cuda_fail(e, "schedule kernel launch");
+}
+
+// The cells take over where nothing asks for another layout.
+static bool all_automatic(const Plan* P)
+{
+    return !P->sched_transport && !P->sched_layout && !P->sched_copy && !P->sched_slices &&
+           !P->sched_rpc && !P->sched_threads;
+}
+
+int schedule_cells_prepare(Plan* P)
+{
+    P->words.ready = false;
+    if (P->m == 0 || !all_automatic(P)) return DPDR_OK;
+    const bool words = schedule_transport(P) == 2;
+    return words ? schedule_words_prepare(P) : DPDR_OK;
+}
+
+// The cells that dpdr_allreduce_schedule (algo 0) runs on, null when it does
+// not.
+const CellPlan* schedule_cells(const Plan* P, int algo)
+{
+    const CellPlan* C = &P->words;
+    return algo == 0 && schedule_transport(P) == 2 && C->ready && all_automatic(P) ? C : nullptr;
+}
+
+}  // namespace dpdr

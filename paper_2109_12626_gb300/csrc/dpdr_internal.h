@@ -57,6 +57,45 @@ struct TreeTables {
     int* levoff = nullptr;
 };
 
+// A subtree cell of the schedule kernels (schedule_cells.cuh): a connected
+// piece of a tree that one warp runs for a column slice.
+constexpr int kWordsRanks = 8, kWordsLevels = 4;
+constexpr int kCellRanks = kWordsRanks;
+constexpr int kCellLevels = kWordsLevels;
+constexpr int kCellExt = kCellRanks / 2;
+struct CellDesc {
+    int n, root, depth;        // ranks, root rank and its depth
+    int par_cell, par_rank;    // the root's parent, -1 at a tree's root
+    int nlev;                  // levels
+    int next;                  // nodes whose two children are roots of other cells
+    int down, par_down;        // number among the cells with next > 0, the parent cell's
+    int reread;                // bit t: the final blocks of position lev_k[t] are read again
+    int rank[kCellRanks];      // post-order, the root last
+    int node_par[kCellRanks];  // parent rank inside the cell, -1 at the root
+    int tape[kCellRanks];      // bits 0-1 children in the cell, 2 child_1 of its parent,
+                               // 3-7 position of its child_1
+    int lev_off[kCellLevels + 1];
+    int lev_k[kCellRanks];     // positions by level, the root first
+    int ext_k[kCellExt];       // positions of the nodes with children elsewhere
+    int ext_cell[2 * kCellExt];  // their children's cells: child_0, child_1 of each
+    int ext_rank[2 * kCellExt];  // and ranks
+};
+
+// Cells of one kind, in one device allocation: control words, descriptors,
+// scratch.
+struct CellPlan {
+    bool ready = false;
+    int n = 0, root0 = -1, root1 = 0;  // cells, the roots' cells (root0 -1: one tree)
+    int down = 0;                      // cells with children in other cells
+    int ranks = 0;                     // of the largest cell
+    int warps = 0;                     // resident warps
+    char* d = nullptr;
+    size_t bytes = 0, off_scratch = 0, scratch = 0;
+};
+struct CellSlices {
+    int n, waves;   // column slices side by side, one after another
+};
+
 struct Plan {
     int p = 0;
     int64_t m = 0;
@@ -114,6 +153,10 @@ struct Plan {
     // words, then the up and down word arrays; own allocation
     char* d_ll = nullptr;
     size_t d_ll_bytes = 0;
+
+    // subtree cells of the schedule kernels, used while every schedule
+    // option is automatic
+    CellPlan words;
 
     // rank-pointer staging (pinned host), copied to d_x / d_y when they change
     const void** h_ptrs = nullptr;   // [2p]
@@ -196,6 +239,17 @@ int fused_tree_index(const Plan* P);            // fused_tree.cu: the device pat
 int schedule_launch(Plan* P, cudaStream_t s,   // schedule.cu: Algorithm 1 (algo 0)
                     int algo = 0);              // or reduce, then broadcast (1)
 int schedule_configure(Plan* P);                // schedule.cu
+// schedule kernels on subtree cells (cells.cpp, schedule_words.cu)
+int schedule_cells_prepare(Plan* P);
+const CellPlan* schedule_cells(const Plan* P, int algo);  // the cells algo runs on, or null
+void make_cells(const Plan* P, int max_ranks, int max_levels, CellPlan* C, std::vector<CellDesc>* out);
+CellSlices cell_slices(const Plan* P, const CellPlan& C, bool vec);
+bool cell_vector(const Plan* P);
+int cell_tail(const Plan* P, bool vec);
+int cell_scratch(Plan* P, CellPlan* C, const void* desc, size_t desc_bytes);
+int cell_launch(const void* kernel, void* args, int64_t warps, int per_cta, size_t smem, cudaStream_t s);
+int schedule_words_prepare(Plan* P);
+int schedule_words_launch(Plan* P, cudaStream_t s);
 int schedule_plan_rpc(Plan* P);                 // schedule.cu: ranks per CTA only
 int schedule_transport(const Plan* P);          // schedule_ll.cu: 1 counters, 2 words
 const void* schedule_ll_kernel_for(int dtype);  // schedule_ll.cu

@@ -259,6 +259,7 @@ static void free_plan(Plan* P)
         if (T.d) cudaFree(T.d);
     if (P->d_sched) cudaFree(P->d_sched);
     if (P->d_ll) cudaFree(P->d_ll);
+    if (P->words.d) cudaFree(P->words.d);
     if (P->h_ptrs) cudaFreeHost(P->h_ptrs);
     if (P->dmem) cudaFree(P->dmem);
     delete P;
@@ -393,7 +394,6 @@ extern "C" dpdr_plan_t dpdr_plan_topo(int p, int64_t m, dpdr_dtype dtype, dpdr_o
     }
     P->b = b == 0 ? default_blocks(P) : clamp_b(m, b);
     if (allocate(P) != DPDR_OK || schedule_configure(P) != DPDR_OK ||
-        (schedule_transport(P) == 2 && schedule_ll_prepare(P) != DPDR_OK) ||
         fused_tree_prepare(P) != DPDR_OK ||  // small; the host path may use it
         fused_split_prepare(P, false, P->split_depth) != DPDR_OK) {
         free_plan(P);
@@ -524,11 +524,12 @@ extern "C" int dpdr_plan_info(dpdr_plan_t h, int64_t* info, int n)
     const int64_t v[] = {P->p, P->m, P->b, P->max_depth, fused_auto_mode(P),
                          P->sched_ctas, P->sched_ranks_per_cta,
                          int64_t(P->dmem_bytes + P->d_split_bytes + P->d_sched_bytes +
-                                 P->d_ll_bytes + P->tree[0].bytes + P->tree[1].bytes),
+                                 P->d_ll_bytes + P->words.bytes + P->tree[0].bytes + P->tree[1].bytes),
                          P->last_vector_path, P->split_s, P->split_nseg, P->split_group,
                          P->sched_slices_used, P->topo, P->last_host_path,
                          schedule_transport(P), P->tree[fused_tree_index(P)].width,
-                         P->sched_layout_used, P->sched_copy_used};
+                         P->sched_layout_used, P->sched_copy_used,
+                         schedule_cells(P, 0) ? schedule_cells(P, 0)->n : 0};
     const int k = int(sizeof v / sizeof v[0]);
     for (int i = 0; i < n; i++) info[i] = i < k ? v[i] : 0;
     return DPDR_OK;

@@ -1159,7 +1159,9 @@ int schedule_configure(Plan* P)
                        cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return cuda_fail(e, "schedule table upload");
     // the automatic transport may have changed with the layout
-    return words ? schedule_ll_prepare(P) : DPDR_OK;
+    rc = schedule_cells_prepare(P);
+    if (rc) return rc;
+    return words && !schedule_cells(P, 0) ? schedule_ll_prepare(P) : DPDR_OK;
 }
 
 int schedule_launch(Plan* P, cudaStream_t s, int algo)

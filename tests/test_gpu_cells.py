@@ -1,0 +1,158 @@
+"""The schedule kernels on subtree cells, which run while every schedule
+option is automatic: bit for bit against the oracle's fold, for both
+topologies.
+
+Sizes are the edges of the cell layout: one cell, cells of one rank, the
+first cut edges (p = 15, 16, 36), ragged last levels; slices of one unit, of
+32, partly filled, several waves of them; blocks that start and end inside a
+16-byte unit or lie within one, rows with a ragged tail."""
+import numpy as np
+import pytest
+import torch
+
+from gpu_util import bits, empty_like_ranks, expect_bits, host_inputs, to_device
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def pkg():
+    from paper_2109_12626_gb300 import build as B
+    B.build()
+    import paper_2109_12626_gb300 as P
+    return P
+
+
+def _dt(orc, kind):
+    return {"int32": orc.I32, "float32": orc.F32, "mat2x2u32": orc.MAT,
+            "mat2x2f32": orc.MATF}[kind]
+
+
+def _buffers(x, kind, layout, dev):
+    pad = 1 if layout == "four_byte" else 0
+    xs, keep = to_device(x, kind, dev, pad_front=pad)
+    if layout == "in_place":
+        return xs, xs, keep
+    ys, keep_y = empty_like_ranks(xs, pad_front=pad)
+    return xs, ys, (keep, keep_y)
+
+
+def _check(ys, want, what):
+    for i, y in enumerate(ys):
+        bad = np.nonzero(bits(y) != want)[0]
+        assert bad.size == 0, "%s rank %d: %d words differ, first %d" % (what, i, bad.size, bad[0])
+
+
+# flagged words between cells: at most 12 MiB of inputs (24 from p = 1024)
+CASES = [("int32", 1, 33, (1, 4)), ("float32", 2, 1, (1,)), ("float32", 2, 4100, (1, 3)),
+         ("int32", 3, 129, (1, 129)), ("mat2x2u32", 7, 300, (1, 7)), ("int32", 15, 1000, (1, 4, 250)),
+         ("float32", 16, 4099, (1, 9, 2000)), ("mat2x2f32", 31, 129, (1, 5)),
+         ("int32", 36, 1003, (1, 3, 400)), ("mat2x2u32", 100, 77, (1, 7)),
+         ("float32", 255, 2050, (1, 16)), ("int32", 288, 250, (1, 2)),
+         ("float32", 1152, 4099, (1, 6)), ("int32", 1152, 1, (1,))]
+
+
+@pytest.mark.parametrize("kind,p,m,blocks", CASES)
+@pytest.mark.parametrize("layout", ["aligned", "in_place", "four_byte"])
+@pytest.mark.parametrize("run", ["dual", "single"])
+def test_cells_match_oracle(pkg, orc, kind, p, m, blocks, layout, run):
+    x = host_inputs(kind, 101, p, m)
+    topo = "dual" if run == "dual" else "single"
+    want = expect_bits(orc.tree_fold(x, _dt(orc, kind), orc.DUAL if topo == "dual" else orc.SINGLE))
+    dev = torch.device("cuda:0")
+    for b in blocks:
+        xs, ys, _keep = _buffers(x, kind, layout, dev)
+        with pkg.Plan(p, m, kind, b, topology=topo) as plan:
+            assert plan.info()["sched_cells"] > 0
+            call = plan.allreduce_reduce_bcast if run == "reduce_bcast" else plan.allreduce_schedule
+            for again in range(1 if layout == "in_place" else 2):
+                call(xs, ys)
+                plan.sync()
+                _check(ys, want, "b=%d call %d" % (b, again))
+        if layout != "in_place":
+            for i in range(p):  # inputs untouched
+                assert np.array_equal(bits(xs[i]), expect_bits(x[i])), i
+
+
+def test_cells_choice(pkg):
+    """On cells while every schedule option is automatic and one slice of
+    them fits the GPU; any option set takes the layouts it names."""
+    for key, value in ((pkg.OPT_SCHED_TRANSPORT, 1), (pkg.OPT_SCHED_TRANSPORT, 2),
+                       (pkg.OPT_SCHED_LAYOUT, 1), (pkg.OPT_SCHED_COPY, 2),
+                       (pkg.OPT_SCHED_SLICES, 2), (pkg.OPT_SCHED_RANKS_PER_CTA, 2),
+                       (pkg.OPT_SCHED_THREADS, 64)):
+        with pkg.Plan(36, 1000, "int32", 3) as plan:
+            assert plan.info()["sched_cells"] > 0
+            plan.set(key, value)
+            assert plan.info()["sched_cells"] == 0
+            plan.set(key, 0)
+            assert plan.info()["sched_cells"] > 0
+    with pkg.Plan(65535, 3, "int32", 1) as plan:
+        assert plan.info()["sched_cells"] == 0
+
+
+@pytest.mark.parametrize("p,m", [(30, 777)], ids=["words"])
+@pytest.mark.parametrize("run", ["schedule"])
+def test_cells_graph_replay(pkg, orc, p, m, run):
+    """Epochs and counter bases move on the device: a captured call replays
+    with new inputs, and plain calls go on between replays."""
+    kind, dev = "int32", torch.device("cuda:0")
+    xs = [torch.empty(m, dtype=torch.int32, device=dev) for _ in range(p)]
+    ys = [torch.empty(m, dtype=torch.int32, device=dev) for _ in range(p)]
+    with pkg.Plan(p, m, kind, 3, topology="single") as plan:
+        bound = plan.bind(xs, ys)
+        call = bound.allreduce_schedule if run == "schedule" else bound.allreduce_reduce_bcast
+        s = torch.cuda.Stream()
+        s.wait_stream(torch.cuda.current_stream())
+        with torch.cuda.stream(s):
+            call()
+        torch.cuda.current_stream().wait_stream(s)
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            call()
+        for seed in (1, 2, 3, 4):
+            x = host_inputs(kind, 110 + seed, p, m, lo=-1000, hi=1000)
+            for i in range(p):
+                xs[i].copy_(torch.from_numpy(x[i]))
+                ys[i].fill_(-7)
+            if seed == 3:
+                call()
+            else:
+                g.replay()
+            torch.cuda.synchronize()
+            _check(ys, expect_bits(orc.tree_fold(x, orc.I32, orc.SINGLE)), "seed %d" % seed)
+        plan.sync()
+
+
+@pytest.mark.parametrize("p,m,b", [(7, 1000, 4), (36, 1000, 1), (1152, 500, 4)])
+@pytest.mark.parametrize("run", ["dual"])
+def test_cells_silent_rank_times_out_and_recovers(pkg, orc, p, m, b, run):
+    """A rank that never publishes -- a leaf, an inner rank of a cell, a
+    cell's root, a tree's root -- makes its partners' waits expire; the plan
+    works again afterwards."""
+    from paper_2109_12626_gb300 import DpdrError
+    kind = "int32"
+    topo = "dual" if run == "dual" else "single"
+    x = host_inputs(kind, 103, p, m, lo=-1000, hi=1000)
+    want = expect_bits(orc.tree_fold(x, orc.I32, orc.DUAL if run == "dual" else orc.SINGLE))
+    xs, _ = to_device(x, kind, torch.device("cuda:0"))
+    with pkg.Plan(p, m, kind, b, topology=topo) as plan:
+        assert plan.info()["sched_cells"] > 0
+        call = plan.allreduce_reduce_bcast if run == "reduce_bcast" else plan.allreduce_schedule
+        plan.set(pkg.OPT_WAIT_LIMIT_NS, 20_000_000)
+        c0 = plan.query()["child0"]
+        ranks = {0, 1, 2, p // 2, p - 2, p - 1} | {int(np.nonzero(c0 >= 0)[0][k]) for k in (0, -2)}
+        if plan.info()["sched_cells"] == 1:
+            ranks.discard(p - 1)  # one cell: nobody waits for its root
+        for skip in sorted(ranks):
+            plan.set(pkg.OPT_SKIP_RANK, skip)
+            ys, _ = empty_like_ranks(xs)
+            call(xs, ys)
+            with pytest.raises(DpdrError) as e:
+                plan.sync()
+            assert e.value.status == pkg.DPDR_ERR_TIMEOUT, skip
+            plan.set(pkg.OPT_SKIP_RANK, -1)
+            call(xs, ys)
+            plan.sync()
+            _check(ys, want, "after %d" % skip)
