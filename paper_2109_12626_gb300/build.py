@@ -24,7 +24,7 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 SOURCES = ["plan.cpp", "api.cpp", "fused.cu", "fused_stream.cu", "fused_tile.cu",
            "fused_split.cu", "fused_bulk.cu", "schedule.cu",
            "schedule_ll.cu", "cells.cpp", "schedule_words.cu",
-           "fused_tree.cu"]
+           "schedule_walk.cu", "schedule_walk_rb.cu", "fused_tree.cu"]
 
 
 def nvcc() -> str:

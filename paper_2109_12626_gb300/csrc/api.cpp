@@ -122,7 +122,8 @@ extern "C" int dpdr_allreduce_schedule(dpdr_plan_t h, const void* const* x,
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     int rc = prepare(P, x, reinterpret_cast<const void* const*>(y), s);
     if (rc) return rc;
-    if (P->m && schedule_cells(P, 0)) return schedule_words_launch(P, s);
+    if (P->m && schedule_cells(P, 0))
+        return schedule_transport(P) == 2 ? schedule_words_launch(P, s) : schedule_walk_launch(P, s, 0);
     return schedule_transport(P) == 2 ? schedule_ll_launch(P, s) : schedule_launch(P, s);
 }
 
@@ -137,7 +138,7 @@ extern "C" int dpdr_allreduce_reduce_bcast(dpdr_plan_t h, const void* const* x,
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     int rc = prepare(P, x, reinterpret_cast<const void* const*>(y), s);
     if (rc) return rc;
-    return schedule_launch(P, s, 1);
+    return P->m && schedule_cells(P, 1) ? schedule_walk_launch(P, s, 1) : schedule_launch(P, s, 1);
 }
 
 // Column chunks of about host_chunk bytes of rank data (default 1 GB), each

@@ -1,6 +1,7 @@
 // cells.cpp -- host side of the schedule kernels on subtree cells: how the
 // trees are cut into cells, the cells' device descriptors, their column
-// slices, scratch and launches (schedule_cells.cuh, schedule_words.cu).
+// slices, scratch and launches (schedule_cells.cuh, schedule_words.cu,
+// schedule_walk.cu).
 #include <algorithm>
 #include <cstring>
 #include <map>
@@ -206,10 +207,12 @@ int cell_scratch(Plan* P, CellPlan* C, const void* desc, size_t desc_bytes)
         }
         C->bytes = bytes;
     }
+    std::vector<char> head(256 + desc_bytes, 0);
     const uint32_t one = 1;
-    e = cudaMemset(C->d, 0, bytes);
-    if (e == cudaSuccess) e = cudaMemcpy(C->d, &one, sizeof one, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(C->d + 256, desc, desc_bytes, cudaMemcpyHostToDevice);
+    std::memcpy(head.data(), &one, sizeof one);
+    std::memcpy(head.data() + 256, desc, desc_bytes);
+    e = cudaMemset(C->d + C->off_scratch, 0, C->scratch);
+    if (e == cudaSuccess) e = cudaMemcpy(C->d, head.data(), head.size(), cudaMemcpyHostToDevice);
     return e == cudaSuccess ? DPDR_OK : cuda_fail(e, "schedule cells: upload");
 }
 
@@ -234,18 +237,20 @@ static bool all_automatic(const Plan* P)
 
 int schedule_cells_prepare(Plan* P)
 {
-    P->words.ready = false;
+    P->words.ready = P->walk.ready = false;
     if (P->m == 0 || !all_automatic(P)) return DPDR_OK;
     const bool words = schedule_transport(P) == 2;
-    return words ? schedule_words_prepare(P) : DPDR_OK;
+    int rc = words ? schedule_words_prepare(P) : DPDR_OK;
+    if (rc == DPDR_OK && (!words || P->topo == DPDR_TOPO_SINGLE)) rc = schedule_walk_prepare(P);
+    return rc;
 }
 
-// The cells that dpdr_allreduce_schedule (algo 0) runs on, null when it does
-// not.
+// The cells that dpdr_allreduce_schedule (algo 0) or
+// dpdr_allreduce_reduce_bcast (1) runs on, null when it does not.
 const CellPlan* schedule_cells(const Plan* P, int algo)
 {
-    const CellPlan* C = &P->words;
-    return algo == 0 && schedule_transport(P) == 2 && C->ready && all_automatic(P) ? C : nullptr;
+    const CellPlan* C = algo == 0 && schedule_transport(P) == 2 ? &P->words : &P->walk;
+    return C->ready && all_automatic(P) ? C : nullptr;
 }
 
 }  // namespace dpdr

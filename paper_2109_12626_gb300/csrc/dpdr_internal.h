@@ -58,10 +58,12 @@ struct TreeTables {
 };
 
 // A subtree cell of the schedule kernels (schedule_cells.cuh): a connected
-// piece of a tree that one warp runs for a column slice.
+// piece of a tree that one warp runs for a column slice.  The largest cells
+// that the kernels take: flagged words, counters.
 constexpr int kWordsRanks = 8, kWordsLevels = 4;
-constexpr int kCellRanks = kWordsRanks;
-constexpr int kCellLevels = kWordsLevels;
+constexpr int kWalkRanks = 20, kWalkLevels = 5;
+constexpr int kCellRanks = kWalkRanks;
+constexpr int kCellLevels = kWalkLevels;
 constexpr int kCellExt = kCellRanks / 2;
 struct CellDesc {
     int n, root, depth;        // ranks, root rank and its depth
@@ -155,8 +157,8 @@ struct Plan {
     size_t d_ll_bytes = 0;
 
     // subtree cells of the schedule kernels, used while every schedule
-    // option is automatic
-    CellPlan words;
+    // option is automatic: flagged words, counters
+    CellPlan words, walk;
 
     // rank-pointer staging (pinned host), copied to d_x / d_y when they change
     const void** h_ptrs = nullptr;   // [2p]
@@ -239,7 +241,8 @@ int fused_tree_index(const Plan* P);            // fused_tree.cu: the device pat
 int schedule_launch(Plan* P, cudaStream_t s,   // schedule.cu: Algorithm 1 (algo 0)
                     int algo = 0);              // or reduce, then broadcast (1)
 int schedule_configure(Plan* P);                // schedule.cu
-// schedule kernels on subtree cells (cells.cpp, schedule_words.cu)
+// schedule kernels on subtree cells (cells.cpp, schedule_words.cu,
+// schedule_walk.cu)
 int schedule_cells_prepare(Plan* P);
 const CellPlan* schedule_cells(const Plan* P, int algo);  // the cells algo runs on, or null
 void make_cells(const Plan* P, int max_ranks, int max_levels, CellPlan* C, std::vector<CellDesc>* out);
@@ -250,6 +253,8 @@ int cell_scratch(Plan* P, CellPlan* C, const void* desc, size_t desc_bytes);
 int cell_launch(const void* kernel, void* args, int64_t warps, int per_cta, size_t smem, cudaStream_t s);
 int schedule_words_prepare(Plan* P);
 int schedule_words_launch(Plan* P, cudaStream_t s);
+int schedule_walk_prepare(Plan* P);
+int schedule_walk_launch(Plan* P, cudaStream_t s, int algo);
 int schedule_plan_rpc(Plan* P);                 // schedule.cu: ranks per CTA only
 int schedule_transport(const Plan* P);          // schedule_ll.cu: 1 counters, 2 words
 const void* schedule_ll_kernel_for(int dtype);  // schedule_ll.cu

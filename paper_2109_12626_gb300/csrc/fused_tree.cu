@@ -23,6 +23,7 @@
 // than 16 bytes per rank) gets one extra CTA that runs the same three
 // phases on them.
 #include <algorithm>
+#include <cstring>
 #include <vector>
 
 #include "fused_common.cuh"
@@ -216,11 +217,11 @@ static int tree_tables(Plan* P, int W, TreeTables* T)
     char* d = nullptr;
     cudaError_t e = cudaMalloc(&d, bytes);
     if (e != cudaSuccess) return cuda_fail(e, "tree layout: cudaMalloc");
-    e = cudaMemcpy(d, seg.data(), sizeof(int2) * seg.size(), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess && !lev.empty())
-        e = cudaMemcpy(d + o_lev, lev.data(), sizeof(int4) * lev.size(), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess)
-        e = cudaMemcpy(d + o_off, off.data(), sizeof(int) * off.size(), cudaMemcpyHostToDevice);
+    std::vector<char> up(bytes, 0);
+    std::memcpy(up.data(), seg.data(), sizeof(int2) * seg.size());
+    if (!lev.empty()) std::memcpy(up.data() + o_lev, lev.data(), sizeof(int4) * lev.size());
+    std::memcpy(up.data() + o_off, off.data(), sizeof(int) * off.size());
+    e = cudaMemcpy(d, up.data(), bytes, cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
         cudaFree(d);
         return cuda_fail(e, "tree layout: upload");

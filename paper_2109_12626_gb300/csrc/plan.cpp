@@ -259,7 +259,8 @@ static void free_plan(Plan* P)
         if (T.d) cudaFree(T.d);
     if (P->d_sched) cudaFree(P->d_sched);
     if (P->d_ll) cudaFree(P->d_ll);
-    if (P->words.d) cudaFree(P->words.d);
+    for (CellPlan* C : {&P->words, &P->walk})
+        if (C->d) cudaFree(C->d);
     if (P->h_ptrs) cudaFreeHost(P->h_ptrs);
     if (P->dmem) cudaFree(P->dmem);
     delete P;
@@ -309,19 +310,17 @@ static int allocate(Plan* P)
     std::copy(P->child0.begin(), P->child0.end(), tab.begin() + p);
     std::copy(P->child1.begin(), P->child1.end(), tab.begin() + 2 * p);
     std::copy(P->depth.begin(), P->depth.end(), tab.begin() + 3 * p);
-    struct Up { void* dst; const void* src; size_t n; } ups[] = {
-        {P->d_tape, P->tape.data(), P->tape.size()},
-        {P->d_levels, P->levels.data(), sizeof(LevelNode) * P->levels.size()},
-        {P->d_level_off, P->level_off.data(), sizeof(int) * P->level_off.size()},
-        {P->d_tables, tab.data(), sizeof(int) * tab.size()},
+    // the tables and the cleared error record lie side by side: one upload
+    std::vector<char> up(o_err + sizeof(uint32_t) * 4 - o_tape, 0);
+    auto put = [&](size_t at, const void* src, size_t n) {
+        if (n) std::memcpy(up.data() + (at - o_tape), src, n);
     };
-    for (auto& u : ups) {
-        if (!u.n) continue;
-        e = cudaMemcpy(u.dst, u.src, u.n, cudaMemcpyHostToDevice);
-        if (e != cudaSuccess) return cuda_fail(e, "dpdr_plan: upload");
-    }
-    e = cudaMemset(P->d_err, 0, sizeof(uint32_t) * 4);
-    if (e != cudaSuccess) return cuda_fail(e, "dpdr_plan: memset");
+    put(o_tape, P->tape.data(), P->tape.size());
+    put(o_lv, P->levels.data(), sizeof(LevelNode) * P->levels.size());
+    put(o_lo, P->level_off.data(), sizeof(int) * P->level_off.size());
+    put(o_tab, tab.data(), sizeof(int) * tab.size());
+    e = cudaMemcpy(base + o_tape, up.data(), up.size(), cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) return cuda_fail(e, "dpdr_plan: upload");
 
     e = cudaHostAlloc(reinterpret_cast<void**>(&P->h_ptrs),
                       sizeof(void*) * 2 * size_t(p), cudaHostAllocDefault);
@@ -524,7 +523,7 @@ extern "C" int dpdr_plan_info(dpdr_plan_t h, int64_t* info, int n)
     const int64_t v[] = {P->p, P->m, P->b, P->max_depth, fused_auto_mode(P),
                          P->sched_ctas, P->sched_ranks_per_cta,
                          int64_t(P->dmem_bytes + P->d_split_bytes + P->d_sched_bytes +
-                                 P->d_ll_bytes + P->words.bytes + P->tree[0].bytes + P->tree[1].bytes),
+                                 P->d_ll_bytes + P->words.bytes + P->walk.bytes + P->tree[0].bytes + P->tree[1].bytes),
                          P->last_vector_path, P->split_s, P->split_nseg, P->split_group,
                          P->sched_slices_used, P->topo, P->last_host_path,
                          schedule_transport(P), P->tree[fused_tree_index(P)].width,

@@ -1113,24 +1113,6 @@ int schedule_configure(Plan* P)
             : blk / 1024;
         G = int(std::max<int64_t>(1, std::min<int64_t>({room, want, 64})));
     }
-    const size_t words_n = (2 * size_t(P->p) * G + 1) * kCtr;
-    const size_t off_first = (words_n * sizeof(uint32_t) + 255) / 256 * 256;
-    const size_t off_groups = (off_first + sizeof(int) * first.size() + 255) / 256 * 256;
-    const size_t off_ranks = off_groups + sizeof(int4) * L.groups.size();
-    const size_t bytes = off_ranks + sizeof(int) * L.ranks.size() + 16;
-    cudaError_t e;
-    if (bytes > P->d_sched_bytes) {
-        if (P->d_sched) cudaFree(P->d_sched);
-        P->d_sched = nullptr;
-        P->d_sched_bytes = 0;
-        e = cudaMalloc(&P->d_sched, bytes);
-        if (e != cudaSuccess) return cuda_fail(e, "schedule counters: cudaMalloc");
-        P->d_sched_bytes = bytes;
-    }
-    P->d_ctrl = reinterpret_cast<uint32_t*>(P->d_sched);
-    P->d_cta_first = reinterpret_cast<int*>(P->d_sched + off_first);
-    P->d_groups = reinterpret_cast<int4*>(P->d_sched + off_groups);
-    P->d_rank_list = reinterpret_cast<int*>(P->d_sched + off_ranks);
     P->sched_slices_used = G;
     P->sched_chunks = nchunks;
     P->sched_ctas = nchunks * G;
@@ -1149,6 +1131,28 @@ int schedule_configure(Plan* P)
         if (es != cudaSuccess) return cuda_fail(es, "schedule shared memory");
     }
     P->sched_ranks_per_cta = words || layout == 1 ? R : L.max_ranks;
+    // on cells, the tables and counters of the layout above are not needed
+    rc = schedule_cells_prepare(P);
+    if (rc) return rc;
+    if (schedule_cells(P, 0) && (P->topo == DPDR_TOPO_DUAL || schedule_cells(P, 1))) return DPDR_OK;
+    const size_t words_n = (2 * size_t(P->p) * G + 1) * kCtr;
+    const size_t off_first = (words_n * sizeof(uint32_t) + 255) / 256 * 256;
+    const size_t off_groups = (off_first + sizeof(int) * first.size() + 255) / 256 * 256;
+    const size_t off_ranks = off_groups + sizeof(int4) * L.groups.size();
+    const size_t bytes = off_ranks + sizeof(int) * L.ranks.size() + 16;
+    cudaError_t e;
+    if (bytes > P->d_sched_bytes) {
+        if (P->d_sched) cudaFree(P->d_sched);
+        P->d_sched = nullptr;
+        P->d_sched_bytes = 0;
+        e = cudaMalloc(&P->d_sched, bytes);
+        if (e != cudaSuccess) return cuda_fail(e, "schedule counters: cudaMalloc");
+        P->d_sched_bytes = bytes;
+    }
+    P->d_ctrl = reinterpret_cast<uint32_t*>(P->d_sched);
+    P->d_cta_first = reinterpret_cast<int*>(P->d_sched + off_first);
+    P->d_groups = reinterpret_cast<int4*>(P->d_sched + off_groups);
+    P->d_rank_list = reinterpret_cast<int*>(P->d_sched + off_ranks);
     e = cudaMemcpy(P->d_cta_first, first.data(), sizeof(int) * first.size(),
                    cudaMemcpyHostToDevice);
     if (e == cudaSuccess && !L.groups.empty())
@@ -1159,8 +1163,6 @@ int schedule_configure(Plan* P)
                        cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return cuda_fail(e, "schedule table upload");
     // the automatic transport may have changed with the layout
-    rc = schedule_cells_prepare(P);
-    if (rc) return rc;
     return words && !schedule_cells(P, 0) ? schedule_ll_prepare(P) : DPDR_OK;
 }
 

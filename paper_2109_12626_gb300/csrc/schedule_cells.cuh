@@ -1,6 +1,7 @@
 // schedule_cells.cuh -- device pieces shared by the schedule kernels that
-// gather the virtual ranks into subtree cells (schedule_words.cu: flagged
-// words between cells, short blocks).
+// gather the virtual ranks into subtree cells: flagged words between cells
+// for short blocks (schedule_words.cu), counters for large ones
+// (schedule_walk.cu).
 //
 // A cell is a connected piece of a post-order tree.  One warp runs a cell
 // for one column slice of every block, and every lane owns the same columns

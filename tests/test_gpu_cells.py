@@ -1,6 +1,7 @@
 """The schedule kernels on subtree cells, which run while every schedule
 option is automatic: bit for bit against the oracle's fold, for both
-topologies.
+transports between cells (flagged words for small inputs, counters beyond),
+both entry points and both topologies.
 
 Sizes are the edges of the cell layout: one cell, cells of one rank, the
 first cut edges (p = 15, 16, 36), ragged last levels; slices of one unit, of
@@ -50,11 +51,16 @@ CASES = [("int32", 1, 33, (1, 4)), ("float32", 2, 1, (1,)), ("float32", 2, 4100,
          ("int32", 36, 1003, (1, 3, 400)), ("mat2x2u32", 100, 77, (1, 7)),
          ("float32", 255, 2050, (1, 16)), ("int32", 288, 250, (1, 2)),
          ("float32", 1152, 4099, (1, 6)), ("int32", 1152, 1, (1,))]
+# counters between cells
+CASES += [("int32", 2, 1600001, (1, 5)), ("float32", 7, 500003, (1, 8, 600)),
+          ("mat2x2u32", 36, 30001, (1, 7)), ("int32", 100, 40009, (1, 16, 5000)),
+          ("float32", 288, 21250, (0, 1, 3)), ("mat2x2f32", 288, 3001, (4,)),
+          ("int32", 1152, 8193, (0, 1, 5, 1000)), ("float32", 2600, 2051, (0, 3)), ("float32", 2600, 37, (1, 3))]
 
 
 @pytest.mark.parametrize("kind,p,m,blocks", CASES)
 @pytest.mark.parametrize("layout", ["aligned", "in_place", "four_byte"])
-@pytest.mark.parametrize("run", ["dual", "single"])
+@pytest.mark.parametrize("run", ["dual", "single", "reduce_bcast"])
 def test_cells_match_oracle(pkg, orc, kind, p, m, blocks, layout, run):
     x = host_inputs(kind, 101, p, m)
     topo = "dual" if run == "dual" else "single"
@@ -91,8 +97,32 @@ def test_cells_choice(pkg):
         assert plan.info()["sched_cells"] == 0
 
 
-@pytest.mark.parametrize("p,m", [(30, 777)], ids=["words"])
-@pytest.mark.parametrize("run", ["schedule"])
+def test_cells_change_of_options_and_alignment(pkg, orc):
+    """One plan, calls of different kinds in a row: aligned and unaligned
+    buffers (other slice counts over the same counters), other block counts,
+    both entry points, options set and taken back."""
+    kind, p, m = "float32", 100, 40009
+    x = host_inputs(kind, 102, p, m)
+    want = expect_bits(orc.tree_fold(x, orc.F32, orc.SINGLE))
+    dev = torch.device("cuda:0")
+    xa, _ = to_device(x, kind, dev)
+    xu, _keep = to_device(x, kind, dev, pad_front=1)
+    with pkg.Plan(p, m, kind, 4, topology="single") as plan:
+        for step in range(12):
+            if step == 4:
+                plan.set(pkg.OPT_BLOCKS, 37)
+            if step in (6, 9):
+                plan.set(pkg.OPT_SCHED_TRANSPORT, 1 if step == 6 else 0)
+            xs = xu if step % 2 else xa
+            ys, _k = empty_like_ranks(xs, pad_front=step % 2)
+            call = plan.allreduce_reduce_bcast if step % 3 == 2 else plan.allreduce_schedule
+            call(xs, ys)
+            plan.sync()
+            _check(ys, want, "step %d" % step)
+
+
+@pytest.mark.parametrize("p,m", [(30, 777), (100, 40009)], ids=["words", "counters"])
+@pytest.mark.parametrize("run", ["schedule", "reduce_bcast"])
 def test_cells_graph_replay(pkg, orc, p, m, run):
     """Epochs and counter bases move on the device: a captured call replays
     with new inputs, and plain calls go on between replays."""
@@ -125,8 +155,8 @@ def test_cells_graph_replay(pkg, orc, p, m, run):
         plan.sync()
 
 
-@pytest.mark.parametrize("p,m,b", [(7, 1000, 4), (36, 1000, 1), (1152, 500, 4)])
-@pytest.mark.parametrize("run", ["dual"])
+@pytest.mark.parametrize("p,m,b", [(7, 1000, 4), (36, 1000, 1), (1152, 500, 4), (100, 40009, 5)])
+@pytest.mark.parametrize("run", ["dual", "reduce_bcast"])
 def test_cells_silent_rank_times_out_and_recovers(pkg, orc, p, m, b, run):
     """A rank that never publishes -- a leaf, an inner rank of a cell, a
     cell's root, a tree's root -- makes its partners' waits expire; the plan
