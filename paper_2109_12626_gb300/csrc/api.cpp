@@ -54,14 +54,19 @@ static int check_buffers(const Plan* P, const void* const* x,
     return DPDR_OK;
 }
 
+// Whether the device table holds these rank pointers.
+static bool staged(const Plan* P, const void* const* x, const void* const* y)
+{
+    const size_t bytes = sizeof(void*) * size_t(P->p);
+    return P->staged_pending && !std::memcmp(P->last_x.data(), x, bytes) &&
+           !std::memcmp(P->last_y.data(), y, bytes);
+}
+
 int stage_pointers(Plan* P, const void* const* x, const void* const* y,
                    cudaStream_t s)
 {
     const int p = P->p;
-    bool same = true;
-    for (int i = 0; i < p && same; i++)
-        same = P->last_x[i] == x[i] && P->last_y[i] == y[i];
-    if (same && P->staged_pending) return DPDR_OK;  // device table is current
+    if (staged(P, x, y)) return DPDR_OK;  // device table is current
     cudaError_t e;
     if (P->staged_pending) {  // the previous upload must have left the buffer
         e = cudaEventSynchronize(P->staged);
@@ -86,12 +91,7 @@ static int prepare(Plan* P, const void* const* x, const void* const* y,
                    cudaStream_t s)
 {
     if (!x || !y) return fail(DPDR_ERR_INVALID, "x or y is NULL");
-    if (P->staged_pending) {  // same buffers as the last checked call: nothing to do
-        bool same = true;
-        for (int i = 0; i < P->p && same; i++)
-            same = P->last_x[i] == x[i] && P->last_y[i] == y[i];
-        if (same) return DPDR_OK;
-    }
+    if (staged(P, x, y)) return DPDR_OK;  // same buffers as the last checked call
     int vec = 0;
     int rc = check_buffers(P, x, y, &vec);
     if (rc) return rc;
