@@ -151,10 +151,13 @@ int dpdr_plan_query(dpdr_plan_t plan, int* parent, int* child0, int* child1,
  *                             tile, 3 subtree split, 4 bulk-copy pipeline,
  *                             5 hierarchical tile (the five layouts of
  *                             dpdr_allreduce; 3 needs p >= 2 and keeps
- *                             m * esize bytes of scratch per subtree; 4 and
- *                             5 need 16-byte aligned buffers: otherwise 4
- *                             runs as 1, and 5 as 2, or as 3 (else 1) when
- *                             a tile row of p elements does not fit)
+ *                             m * esize bytes of scratch per subtree; 4,
+ *                             and for matrices 5, need 16-byte aligned
+ *                             buffers: otherwise 4 runs as 1, and 5 as 2,
+ *                             or as 3 (else 1) when a tile row of p
+ *                             elements does not fit; the automatic choice
+ *                             may differ for buffers of 4-byte elements
+ *                             that are not 16-byte aligned)
  *   DPDR_OPT_WAIT_LIMIT_NS    bound of every wait of the schedule kernel,
  *                             nanoseconds: 1e3 .. 1e10 (default 4e9); values
  *                             outside that range are DPDR_ERR_INVALID, so a

@@ -168,10 +168,10 @@ struct Plan {
 
     // dynamic shared memory already granted to the fused kernels of this
     // plan's element type (stream, tile, split, bulk, hierarchical tile of
-    // either width, paired stream), so
+    // either width, paired stream; then the same on unaligned rows), so
     // launches skip the attribute call; the limits themselves only ever rise
-    int smem_attr[7] = {48 * 1024, 48 * 1024, 48 * 1024, 48 * 1024, 48 * 1024, 48 * 1024,
-                        48 * 1024};
+    int smem_attr[14] = {48 * 1024, 48 * 1024, 48 * 1024, 48 * 1024, 48 * 1024, 48 * 1024, 48 * 1024,
+                         48 * 1024, 48 * 1024, 48 * 1024, 48 * 1024, 48 * 1024, 48 * 1024, 48 * 1024};
 
     // split layout of the fused kernel (fused.cu): subtrees at depth split_s
     bool split_ready = false;

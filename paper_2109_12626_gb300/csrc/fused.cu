@@ -158,6 +158,20 @@ int fused_auto_mode(const Plan* P)
     return P->split_ready ? 3 : 1;
 }
 
+// On rows of 4-byte elements that are only 4-byte aligned the shared-memory
+// tile copies word by word, so the layouts beside it take over earlier
+// (graph replays, int32): the hierarchical tile in deep trees (p = 288,
+// m = 1001 in 7.1 against 7.9 us, m = 21250 21.2 against 23.5; p = 192,
+// m = 32769 18.3 against 21.4; p = 1152, m = 4099 19.1 against 23.5, but
+// m = 1023 16.4 against 15.4), column streaming from half the columns (p = 64,
+// m = 65537 14.0 against 15.5).
+static int unaligned_mode(const Plan* P)
+{
+    const int64_t units = P->m * int64_t(P->esize) / 16;
+    if (P->p >= 128) return units >= (P->p >= 1024 ? 1024 : 128) ? 5 : 2;
+    return units >= stream_target(P) / 10 ? 1 : 2;
+}
+
 // Whether the automatic choice can be the split layout (then the plan
 // prepares it up front).
 static bool split_wanted(const Plan* P)
@@ -262,18 +276,19 @@ int fused_launch_cols(Plan* P, const char* const* dx, char* const* dy, int64_t m
     if (mc == 0) return DPDR_OK;
     int mode = force_mode ? force_mode : P->fused_mode ? P->fused_mode : fused_auto_mode(P);
     const int lg = tile_lg_wu(P);
+    const bool quad = !vec && P->esize == 4;
+    if (quad && !force_mode && !P->fused_mode && mode == 2) mode = unaligned_mode(P);
     if (mode == 2 && lg < 0) return fail(DPDR_ERR_INVALID, "tile mode: p too large");
     if (mode == 3 && !P->split_ready) return fail(DPDR_ERR_INVALID, "split mode: p < 2");
     const TreeTables& T = P->tree[tree_index < 0 ? fused_tree_index(P) : tree_index];
     if (mode == 5 && !T.ready) return fail(DPDR_ERR_INVALID, "tree mode not prepared");
     if (mode < 1 || mode > 5) return fail(DPDR_ERR_INVALID, "unknown fused mode");
-    // the bulk and hierarchical layouts need 16-byte rows: without them the
-    // bulk layout's work goes to column streaming, the hierarchical tile's to
-    // the shared-memory tile (or, when a tile row does not fit, the split
-    // layout), which keep its short walks (p = 288, m = 21250 int32 with
-    // rows 8 bytes apart from 16: 22.8 against 57 us streamed)
+    // the bulk layout needs 16-byte rows, the hierarchical one units of 16
+    // bytes: without them the bulk layout's work goes to column streaming, the
+    // hierarchical tile's (matrices) to the shared-memory tile (or, when a
+    // tile row does not fit, the split layout), which keep its short walks
     if (mode == 4 && !vec) mode = 1;
-    if (mode == 5 && !vec) mode = lg >= 0 ? 2 : P->split_ready ? 3 : 1;
+    if (mode == 5 && !vec && !quad) mode = lg >= 0 ? 2 : P->split_ready ? 3 : 1;
 
     FusedArgs a;
     a.x = dx;
@@ -287,7 +302,9 @@ int fused_launch_cols(Plan* P, const char* const* dx, char* const* dy, int64_t m
     a.r1 = P->r1;
     a.dual = P->r0 >= 0 ? 1 : 0;
     const int epv = int(16 / P->esize);
-    a.nvec = vec ? mc / epv : 0;
+    a.quad = quad ? 1 : 0;
+    const int64_t group = mode == 5 ? T.width : mode == 2 ? fused::kQuadTile : fused::kQuadStream;
+    a.nvec = quad ? mc / (4 * group) * group : vec ? mc / epv : 0;
     a.scalar_base = a.nvec * epv;
     a.nscalar = mc - a.scalar_base;
     a.lg_wu = lg < 0 ? 0 : lg;

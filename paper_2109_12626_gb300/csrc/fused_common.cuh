@@ -46,7 +46,8 @@ struct FusedArgs {
     int p;
     int r0, r1;
     int dual;               // 1: y = v(r0) (.) v(r1); 0: one tree, y = v(p-1)
-    int64_t nvec;           // 16-byte units
+    int64_t nvec;           // 16-byte units, or (quad) units of four single elements
+    int quad;               // rows are not all 16-byte aligned: QuadUnit instead of VecUnit
     int64_t nscalar;        // single elements after the vector units
     int64_t scalar_base;    // element index of the first single element
     int lg_wu;              // tile: log2 of vector units per row
@@ -94,6 +95,74 @@ struct VecUnit {
         st_l2(row + u * 16, v);
     }
 };
+
+// Four 4-byte elements of rows that are only 4-byte aligned: columns c, c + G,
+// c + 2G and c + 3G of a group of 4G, so that G neighbouring units move 4G
+// contiguous elements, in four accesses of 4G contiguous bytes.  G is the
+// units that run side by side on one row: a warp's 32 in the streaming and
+// split layouts, the tile's width in the others.  One element per thread and
+// row left a quarter of the bytes in flight: p = 11, m = 6264977 int32 in
+// 136 us, 87 with these units (83 with aligned rows); p = 62, m = 1862471
+// 206 and 157 (153); p = 1152, m = 65537 163 and 115 (108).
+template <class Op, int G>
+struct QuadUnit {
+    using T = uint4;
+    static constexpr int kStep = 4 * G;  // bytes from one element to the next
+    __device__ __forceinline__ static int64_t at(int64_t u)
+    {
+        return (u / G * (4 * G) + u % G) * 4;
+    }
+    __device__ __forceinline__ static uint32_t ld1(const char* p)
+    {
+        return __ldcs(reinterpret_cast<const unsigned int*>(p));
+    }
+    __device__ __forceinline__ static void st1(char* p, uint32_t v)
+    {
+        __stcs(reinterpret_cast<unsigned int*>(p), v);
+    }
+    __device__ __forceinline__ static T ld(const char* row, int64_t u)
+    {
+        const char* p = row + at(u);
+        return make_uint4(ld1(p), ld1(p + kStep), ld1(p + 2 * kStep), ld1(p + 3 * kStep));
+    }
+    __device__ __forceinline__ static void st(char* row, int64_t u, const T& v)
+    {
+        char* p = row + at(u);
+        st1(p, v.x);
+        st1(p + kStep, v.y);
+        st1(p + 2 * kStep, v.z);
+        st1(p + 3 * kStep, v.w);
+    }
+    __device__ __forceinline__ static T op(const T& a, const T& b) { return Op::vec(a, b); }
+    __device__ __forceinline__ static T ld_keep(const char* row, int64_t u)
+    {
+        const char* p = row + at(u);
+        return make_uint4(ld_l2_u32(p), ld_l2_u32(p + kStep), ld_l2_u32(p + 2 * kStep),
+                          ld_l2_u32(p + 3 * kStep));
+    }
+    __device__ __forceinline__ static void st_keep(char* row, int64_t u, const T& v)
+    {
+        char* p = row + at(u);
+        st_l2_u32(p, v.x);
+        st_l2_u32(p + kStep, v.y);
+        st_l2_u32(p + 2 * kStep, v.z);
+        st_l2_u32(p + 3 * kStep, v.w);
+    }
+};
+
+// The wide unit of a launch: 16-byte units, or on unaligned rows of 4-byte
+// elements (a.quad) four of them; f is called with a value of the unit type.
+template <class Op, int G, class F>
+inline int with_unit(const FusedArgs& a, F f)
+{
+    if constexpr (Op::kEpv == 4) {
+        if (a.quad) return f(QuadUnit<Op, G>());
+    }
+    return f(VecUnit<Op>());
+}
+constexpr int kQuadStream = 32;  // G of the streaming and split layouts
+constexpr int kQuadTile = 8;     // of the shared-memory tile (as many units or more to a row)
+constexpr int kQuadAttr = 7;  // offset of the unaligned kernels in Plan::smem_attr
 
 template <class Op>
 struct OneUnit {

@@ -71,14 +71,14 @@ __device__ __forceinline__ void split_finish_column(const FusedArgs& a, int r, i
     for (int i = r * a.group; i < i1; i++) U::st(rank_ptr_w(a.y, i), u, y);
 }
 
-template <class Op>
+template <class Op, class V>
 __global__ void __launch_bounds__(kStreamThreads, 4)
 fused_split_reduce_kernel(FusedArgs a)
 {
     extern __shared__ uint4 smem[];
     const int64_t u = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     if (u < a.nvec) {
-        split_reduce_column<VecUnit<Op>>(a, blockIdx.y, u, smem + threadIdx.x, blockDim.x);
+        split_reduce_column<V>(a, blockIdx.y, u, smem + threadIdx.x, blockDim.x);
     } else if (u < a.nvec + a.nscalar) {
         split_reduce_column<OneUnit<Op>>(a, blockIdx.y, a.scalar_base + (u - a.nvec),
                                          one_slots<Op>(smem, threadIdx.x),
@@ -86,14 +86,14 @@ fused_split_reduce_kernel(FusedArgs a)
     }
 }
 
-template <class Op>
+template <class Op, class V>
 __global__ void __launch_bounds__(kStreamThreads, 4)
 fused_split_finish_kernel(FusedArgs a)
 {
     extern __shared__ uint4 smem[];
     const int64_t u = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     if (u < a.nvec) {
-        split_finish_column<VecUnit<Op>>(a, blockIdx.y, u, smem + threadIdx.x, blockDim.x);
+        split_finish_column<V>(a, blockIdx.y, u, smem + threadIdx.x, blockDim.x);
     } else if (u < a.nvec + a.nscalar) {
         split_finish_column<OneUnit<Op>>(a, blockIdx.y, a.scalar_base + (u - a.nvec),
                                          one_slots<Op>(smem, threadIdx.x),
@@ -110,21 +110,25 @@ struct Split {
         const int64_t blocks = (units + kStreamThreads - 1) / kStreamThreads;
         const size_t smem = size_t(P->max_depth + 1) * kStreamThreads * sizeof(uint4);
         if (blocks > 0x7fffffff) return fail(DPDR_ERR_INVALID, "m too large");
-        if (int(smem) > P->smem_attr[2]) {
-            int granted = P->smem_attr[2];
-            if (int rc = grant_smem(reinterpret_cast<const void*>(&fused_split_reduce_kernel<Op>),
-                                    smem, &granted, "fused split attribute"))
-                return rc;
-            if (int rc = grant_smem(reinterpret_cast<const void*>(&fused_split_finish_kernel<Op>),
-                                    smem, &P->smem_attr[2], "fused split attribute"))
-                return rc;
-        }
-        const int groups = (P->p + a.group - 1) / a.group;
-        fused_split_reduce_kernel<Op>
-            <<<dim3(unsigned(blocks), unsigned(P->split_nseg)), kStreamThreads, smem, s>>>(a);
-        fused_split_finish_kernel<Op>
-            <<<dim3(unsigned(blocks), unsigned(groups)), kStreamThreads, smem, s>>>(a);
-        return launched();
+        return with_unit<Op, kQuadStream>(a, [&](auto unit) {
+            using V = decltype(unit);
+            int* const attr = &P->smem_attr[2 + (a.quad ? kQuadAttr : 0)];
+            if (int(smem) > *attr) {
+                int granted = *attr;
+                if (int rc = grant_smem(reinterpret_cast<const void*>(&fused_split_reduce_kernel<Op, V>),
+                                        smem, &granted, "fused split attribute"))
+                    return rc;
+                if (int rc = grant_smem(reinterpret_cast<const void*>(&fused_split_finish_kernel<Op, V>),
+                                        smem, attr, "fused split attribute"))
+                    return rc;
+            }
+            const int groups = (P->p + a.group - 1) / a.group;
+            fused_split_reduce_kernel<Op, V>
+                <<<dim3(unsigned(blocks), unsigned(P->split_nseg)), kStreamThreads, smem, s>>>(a);
+            fused_split_finish_kernel<Op, V>
+                <<<dim3(unsigned(blocks), unsigned(groups)), kStreamThreads, smem, s>>>(a);
+            return launched();
+        });
     }
 };
 

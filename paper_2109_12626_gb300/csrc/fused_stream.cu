@@ -17,14 +17,14 @@ namespace {
 constexpr int64_t kStreamPairUnitsPerSm = 1024;
 constexpr int kStreamPairMinRanks = 16;
 
-template <class Op>
+template <class Op, class V>
 __global__ void __launch_bounds__(kStreamThreads, 4)
 fused_stream_kernel(FusedArgs a)
 {
     extern __shared__ uint4 smem[];
     const int64_t u = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     if (u < a.nvec) {
-        stream_column<VecUnit<Op>>(a, u, smem + threadIdx.x, blockDim.x);
+        stream_column<V>(a, u, smem + threadIdx.x, blockDim.x);
     } else if (u < a.nvec + a.nscalar) {
         stream_column<OneUnit<Op>>(a, a.scalar_base + (u - a.nvec), one_slots<Op>(smem, threadIdx.x),
                                    one_slot_stride<Op>(blockDim.x));
@@ -86,7 +86,7 @@ __device__ __forceinline__ void stream_half(const FusedArgs& a, int64_t u, int h
 // Lanes 0-15 of a warp walk tree 0 for 16 columns, lanes 16-31 tree 1 for
 // the same columns, so a plan with fewer columns than the GPU keeps in
 // flight gets twice the threads and half the walk per thread.
-template <class Op>
+template <class Op, class V>
 __global__ void __launch_bounds__(kStreamThreads, 4)
 fused_stream_pair_kernel(FusedArgs a)
 {
@@ -95,7 +95,7 @@ fused_stream_pair_kernel(FusedArgs a)
     const int64_t c = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) / 32 * 16 + (lane & 15);
     const unsigned pair = (1u << lane) | (1u << (lane ^ 16));
     if (c < a.nvec) {
-        stream_half<VecUnit<Op>>(a, c, h, pair, smem + threadIdx.x, blockDim.x);
+        stream_half<V>(a, c, h, pair, smem + threadIdx.x, blockDim.x);
     } else if (c < a.nvec + a.nscalar) {
         stream_half<OneUnit<Op>>(a, a.scalar_base + (c - a.nvec), h, pair,
                                  one_slots<Op>(smem, threadIdx.x), one_slot_stride<Op>(blockDim.x));
@@ -115,15 +115,18 @@ struct Stream {
         const int64_t blocks = (threads + kStreamThreads - 1) / kStreamThreads;
         const size_t smem = size_t(P->max_depth + 1) * kStreamThreads * sizeof(uint4);
         if (blocks > 0x7fffffff) return fail(DPDR_ERR_INVALID, "m too large");
-        const void* kern = pairs ? reinterpret_cast<const void*>(&fused_stream_pair_kernel<Op>)
-                                 : reinterpret_cast<const void*>(&fused_stream_kernel<Op>);
-        if (int rc = grant_smem(kern, smem, &P->smem_attr[pairs ? 6 : 0], "fused stream attribute"))
-            return rc;
-        if (pairs)
-            fused_stream_pair_kernel<Op><<<unsigned(blocks), kStreamThreads, smem, s>>>(a);
-        else
-            fused_stream_kernel<Op><<<unsigned(blocks), kStreamThreads, smem, s>>>(a);
-        return launched();
+        return with_unit<Op, kQuadStream>(a, [&](auto unit) {
+            using V = decltype(unit);
+            const void* kern = pairs ? reinterpret_cast<const void*>(&fused_stream_pair_kernel<Op, V>)
+                                     : reinterpret_cast<const void*>(&fused_stream_kernel<Op, V>);
+            int* const granted = &P->smem_attr[(pairs ? 6 : 0) + (a.quad ? kQuadAttr : 0)];
+            if (int rc = grant_smem(kern, smem, granted, "fused stream attribute")) return rc;
+            if (pairs)
+                fused_stream_pair_kernel<Op, V><<<unsigned(blocks), kStreamThreads, smem, s>>>(a);
+            else
+                fused_stream_kernel<Op, V><<<unsigned(blocks), kStreamThreads, smem, s>>>(a);
+            return launched();
+        });
     }
 };
 

@@ -27,10 +27,30 @@ __device__ __forceinline__ void cp_async_wait_all()
     asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;\n" ::: "memory");
 }
 
+// Copies unit u of a row into its place in the tile: 16-byte units with
+// 16-byte cp.async, the others word by word.
+template <class Op>
+__device__ __forceinline__ void tile_copy(VecUnit<Op>, uint4* dst, const char* row, int64_t u)
+{
+    cp_async16(dst, row + u * 16);
+}
+template <class Op, int G>
+__device__ __forceinline__ void tile_copy(QuadUnit<Op, G>, uint4* dst, const char* row, int64_t u)
+{
+    const char* src = row + QuadUnit<Op, G>::at(u);
+#pragma unroll
+    for (int w = 0; w < 4; w++) cp_async4(reinterpret_cast<uint32_t*>(dst) + w, src + 4 * G * w);
+}
+template <class Op>
+__device__ __forceinline__ void tile_copy(OneUnit<Op>, Elem<Op>* dst, const char* row, int64_t e)
+{
+    const char* src = row + e * Op::kEsize;
+#pragma unroll
+    for (int w = 0; w < Op::kEsize / 4; w++) cp_async4(reinterpret_cast<uint32_t*>(dst) + w, src + 4 * w);
+}
+
 // rows of WU units: row i < p holds rank i's tile, row p the result.
-// kVec: 16-byte units copied with 16-byte cp.async; otherwise single
-// elements copied word by word with 4-byte cp.async.
-template <class U, bool kVec, class Op>
+template <class U>
 __device__ __forceinline__ void tile_body(const FusedArgs& a, int64_t u0,
                                           int wu, int lg_wu, typename U::T* tile)
 {
@@ -41,14 +61,7 @@ __device__ __forceinline__ void tile_body(const FusedArgs& a, int64_t u0,
     for (int idx = tid; idx < n; idx += bd) {
         const int i = idx >> lg_wu, c = idx & (WU - 1);
         if (c < wu) {
-            if constexpr (kVec) {
-                cp_async16(&tile[idx], rank_ptr(a.x, i) + (u0 + c) * 16);
-            } else {
-                const char* src = rank_ptr(a.x, i) + (u0 + c) * Op::kEsize;
-                uint32_t* dst = reinterpret_cast<uint32_t*>(&tile[idx]);
-#pragma unroll
-                for (int w = 0; w < Op::kEsize / 4; w++) cp_async4(dst + w, src + 4 * w);
-            }
+            tile_copy(U(), &tile[idx], rank_ptr(a.x, i), u0 + c);
         }
     }
     cp_async_wait_all();
@@ -86,7 +99,7 @@ __device__ __forceinline__ int ceil_lg(int w)
     return lg;
 }
 
-template <class Op>
+template <class Op, class V>
 __global__ void __launch_bounds__(kTileThreads)
 fused_tile_kernel(FusedArgs a)
 {
@@ -97,15 +110,14 @@ fused_tile_kernel(FusedArgs a)
     if (t < a.vec_tiles) {
         const int64_t u0 = t << a.lg_wu;
         const int wu = int(lmin(int64_t(1) << a.lg_wu, a.nvec - u0));
-        tile_body<VecUnit<Op>, true, Op>(a, u0, wu, ceil_lg(wu), smem);
+        tile_body<V>(a, u0, wu, ceil_lg(wu), smem);
     } else {
         // single elements: a row of a tile holds as many bytes as in the
         // vector tiles, i.e. 16/esize times more units
         const int lg = a.lg_wu + (Op::kEsize == 4 ? 2 : 0);
         const int64_t e0 = (t - a.vec_tiles) << lg;
         const int wu = int(lmin(int64_t(1) << lg, a.nscalar - e0));
-        tile_body<OneUnit<Op>, false, Op>(a, a.scalar_base + e0, wu, ceil_lg(wu),
-                                          reinterpret_cast<Elem<Op>*>(smem));
+        tile_body<OneUnit<Op>>(a, a.scalar_base + e0, wu, ceil_lg(wu), reinterpret_cast<Elem<Op>*>(smem));
     }
 }
 
@@ -119,11 +131,14 @@ struct Tile {
         const int64_t scal_tiles = (a.nscalar + (int64_t(1) << lg_s) - 1) >> lg_s;
         const int64_t blocks = a.vec_tiles + scal_tiles;
         if (blocks > 0x7fffffff) return fail(DPDR_ERR_INVALID, "m too large");
-        if (int rc = grant_smem(reinterpret_cast<const void*>(&fused_tile_kernel<Op>), smem,
-                                &P->smem_attr[1], "fused tile attribute"))
-            return rc;
-        fused_tile_kernel<Op><<<unsigned(blocks), kTileThreads, smem, s>>>(a);
-        return launched();
+        return with_unit<Op, kQuadTile>(a, [&](auto unit) {
+            using V = decltype(unit);
+            if (int rc = grant_smem(reinterpret_cast<const void*>(&fused_tile_kernel<Op, V>), smem,
+                                    &P->smem_attr[1 + (a.quad ? kQuadAttr : 0)], "fused tile attribute"))
+                return rc;
+            fused_tile_kernel<Op, V><<<unsigned(blocks), kTileThreads, smem, s>>>(a);
+            return launched();
+        });
     }
 };
 

@@ -18,12 +18,15 @@
 // layout pays for a second kernel and a top fold per store group.  A CTA
 // reads all p rows of its columns before it writes any (barrier between
 // phases 1 and 3), and no other CTA touches those columns, so in-place use
-// is safe.  Buffers that are not all 16-byte aligned go to the
-// shared-memory tile (fused.cu); a ragged tail of single elements (fewer
-// than 16 bytes per rank) gets one extra CTA that runs the same three
-// phases on them.
+// is safe.  Rows of 4-byte elements that are only 4-byte aligned take
+// units of four elements apart (QuadUnit, G = W); matrix rows that are not
+// 16-byte aligned go to the shared-memory tile (fused.cu).  A ragged tail of
+// single elements (fewer than 16 bytes per rank; on unaligned rows fewer
+// than 4 W elements) gets extra CTAs, one per W elements, that run the same
+// three phases on them.
 #include <algorithm>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 #include "fused_common.cuh"
@@ -56,8 +59,8 @@ __device__ __forceinline__ typename U::T walk_subtree(const FusedArgs& a, int lo
     return acc;
 }
 
-// The three phases for wu <= W units starting at u0 (16-byte units with
-// VecUnit, single elements with OneUnit); slot/stride are this thread's
+// The three phases for wu <= W units starting at u0 (wide units with
+// VecUnit or QuadUnit, single elements with OneUnit); slot/stride are this thread's
 // walk slots.
 template <class U, int W>
 __device__ __forceinline__ void tree_body(const FusedArgs& a, int64_t u0, int wu, uint4* smem,
@@ -110,7 +113,7 @@ __device__ __forceinline__ void tree_body(const FusedArgs& a, int64_t u0, int wu
 
 // W column units per CTA: kTreeUnitsNarrow for few columns (more CTAs),
 // kTreeUnitsWide for more (longer rows per rank, half the CTAs).
-template <class Op, int W>
+template <class Op, class V, int W>
 __global__ void __launch_bounds__(kTreeThreads, 2)
 fused_tree_kernel(FusedArgs a)
 {
@@ -118,10 +121,10 @@ fused_tree_kernel(FusedArgs a)
     const int tid = threadIdx.x;
     if (blockIdx.x < a.tree_tiles) {
         const int64_t u0 = int64_t(blockIdx.x) * W;
-        tree_body<VecUnit<Op>, W>(a, u0, int(lmin(W, a.nvec - u0)), smem, smem + tid,
-                                  kTreeThreads);
-    } else {  // ragged tail: the single elements after the 16-byte units
-        tree_body<OneUnit<Op>, W>(a, a.scalar_base, int(a.nscalar), smem,
+        tree_body<V, W>(a, u0, int(lmin(W, a.nvec - u0)), smem, smem + tid, kTreeThreads);
+    } else {  // ragged tail: the single elements after the wide units
+        const int64_t e0 = (int64_t(blockIdx.x) - a.tree_tiles) * W;
+        tree_body<OneUnit<Op>, W>(a, a.scalar_base + e0, int(lmin(W, a.nscalar - e0)), smem,
                                   one_slots<Op>(smem, tid), one_slot_stride<Op>(kTreeThreads));
     }
 }
@@ -137,18 +140,21 @@ struct Tree {
     static int run(Plan* P, FusedArgs a, cudaStream_t s)
     {
         const size_t smem = tree_smem(a);
-        const int64_t blocks = a.tree_tiles + (a.nscalar ? 1 : 0);
+        const int64_t blocks = a.tree_tiles + (a.nscalar + a.tree_width - 1) / a.tree_width;
         if (blocks > 0x7fffffff) return fail(DPDR_ERR_INVALID, "m too large");
         const bool wide = a.tree_width == kTreeUnitsWide;
-        const void* kern = wide ? reinterpret_cast<const void*>(&fused_tree_kernel<Op, kTreeUnitsWide>)
-                                : reinterpret_cast<const void*>(&fused_tree_kernel<Op, kTreeUnitsNarrow>);
-        if (int rc = grant_smem(kern, smem, &P->smem_attr[wide ? 5 : 4], "fused tree attribute"))
-            return rc;
-        if (wide)
-            fused_tree_kernel<Op, kTreeUnitsWide><<<unsigned(blocks), kTreeThreads, smem, s>>>(a);
-        else
-            fused_tree_kernel<Op, kTreeUnitsNarrow><<<unsigned(blocks), kTreeThreads, smem, s>>>(a);
-        return launched();
+        auto launch = [&](auto unit, auto width) {
+            using V = decltype(unit);
+            constexpr int W = decltype(width)::value;
+            const void* kern = reinterpret_cast<const void*>(&fused_tree_kernel<Op, V, W>);
+            int* const granted = &P->smem_attr[(wide ? 5 : 4) + (a.quad ? kQuadAttr : 0)];
+            if (int rc = grant_smem(kern, smem, granted, "fused tree attribute")) return rc;
+            fused_tree_kernel<Op, V, W><<<unsigned(blocks), kTreeThreads, smem, s>>>(a);
+            return launched();
+        };
+        constexpr int N = kTreeUnitsNarrow, W = kTreeUnitsWide;
+        return wide ? with_unit<Op, W>(a, [&](auto u) { return launch(u, std::integral_constant<int, W>()); })
+                    : with_unit<Op, N>(a, [&](auto u) { return launch(u, std::integral_constant<int, N>()); });
     }
 };
 
