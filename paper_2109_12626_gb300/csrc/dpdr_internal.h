@@ -95,7 +95,8 @@ struct CellPlan {
     size_t bytes = 0, off_scratch = 0, scratch = 0;
 };
 struct CellSlices {
-    int n, waves;   // column slices side by side, one after another
+    int n, per_block;  // column slices side by side, of a block
+    int steps;         // slices that a warp runs, one after another
 };
 
 struct Plan {

@@ -131,17 +131,18 @@ struct Unit<Op, false> {
     }
 };
 
-// Column slices of 32 units: a warp serves slice g of the first wave,
-// g + nslices of the second and so on, each an independent copy of the
-// schedule; step t runs block t % b of wave t / b, so the next wave's first
-// rounds run while the last wave's final blocks are on their way down.
+// Column slices of 32 units, numbered through all blocks (per_block to a
+// block): in step t warp g of a cell runs slice t nslices + g, so the blocks
+// pass in their order, and every slice through the same warp of each cell.
+// The schedule's rounds are the warp's steps: an exchange that Algorithm 1
+// puts d rounds after another comes d steps after it.
 // With 16-byte units the bounds of the blocks are rounded up to whole units
 // (a block is then up to 3 elements longer or shorter than the partition
 // says); the row's last elements that fill no unit are one more slice of one
 // block, run element by element (tail).
 struct Columns {
     int64_t m, q, rem;   // elements, block partition
-    int b, nslices, waves;
+    int b, nslices, per_block, steps;
     int tail;            // 1: there is a tail slice (the last one)
 };
 
@@ -151,15 +152,14 @@ struct Spot {
     bool on;
 };
 
-// Block and slice of a step, moved on from one step to the next.
+// Block and slice of a step, moved on from one step to the next; past the
+// last block in the last step of some warps (an empty extent).
 struct Pos {
     int j, g;
+    __device__ __forceinline__ Pos(const Columns& c, int slice) : j(slice / c.per_block), g(slice % c.per_block) {}
     __device__ __forceinline__ void advance(const Columns& c)
     {
-        if (++j == c.b) {
-            j = 0;
-            g += c.nslices;
-        }
+        for (g += c.nslices; g >= c.per_block; g -= c.per_block) j++;
     }
 };
 
@@ -184,7 +184,7 @@ __device__ __forceinline__ Extent extent(const Columns& c, const Pos& at, bool t
         }
         u += int64_t(at.g) * 32;
     }
-    return Extent{u, u < e ? int(lmin(e - u, 32)) : 0};
+    return Extent{u, u < e && (tail || at.j < c.b) ? int(lmin(e - u, 32)) : 0};
 }
 template <class Op, bool kVec>
 __device__ __forceinline__ Spot spot(const Columns& c, const Pos& at, int lane, bool tail)

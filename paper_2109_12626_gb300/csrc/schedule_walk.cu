@@ -21,9 +21,9 @@ int schedule_walk_prepare(Plan* P)
     CellPlan& C = P->walk;
     C.ready = false;
     // Cells of at most 16 ranks, and of up to 20 where that takes a whole tree
-    // (p = 36: two cells of 18 ranks, m = 2^20 2x2 matrices in 250 against
+    // (p = 36: two cells of 18 ranks, m = 2^20 2x2 matrices in 231 against
     // 329 us with six; with larger trees 20 ranks make the longest walk
-    // longer: p = 1152, m = 2^16 int32 in 198 against 170 us).
+    // longer: p = 1152, m = 2^16 int32 15 % slower).
     const int tree = P->r0 >= 0 ? P->p - P->p / 2 : P->p;
     std::vector<CellDesc> desc;
     make_cells(P, tree <= walk::kRanks ? walk::kRanks : 16, walk::kLevels, &C, &desc);
@@ -61,7 +61,7 @@ int schedule_walk_launch(Plan* P, cudaStream_t s, int algo)
     a.ctl = reinterpret_cast<uint32_t*>(C.d);
     a.err = P->d_err;
     const CellSlices S = cell_slices(P, C, vec);
-    a.col = cells::Columns{P->m, P->m / P->b, P->m % P->b, P->b, S.n, S.waves, cell_tail(P, vec)};
+    a.col = cells::Columns{P->m, P->m / P->b, P->m % P->b, P->b, S.n, S.per_block, S.steps, cell_tail(P, vec)};
     const int64_t warps = int64_t(C.n) * (S.n + a.col.tail);
     // counters of all geometries share one array, so that clearing it once
     // clears what another geometry left; the exchange slots lie behind it
@@ -75,7 +75,7 @@ int schedule_walk_launch(Plan* P, cudaStream_t s, int algo)
     a.root0 = C.root0;
     a.root1 = C.root1;
     a.ranks = C.ranks;
-    a.used = P->b * S.waves + P->max_depth + 2;
+    a.used = S.steps + P->max_depth + 2;
     a.skip_rank = P->skip_rank;
     return cell_launch(kernel(P->dtype, vec, algo), &a, warps, walk::kWarps,
                        walk::smem_for(C.ranks), s);

@@ -13,15 +13,14 @@
 // and partial blocks, the fold, a release fence, the parent's counter and
 // final block, the stores, another fence -- and device memory.  24 warps per
 // SM, each with its next step's inputs on their way into shared memory
-// (cp.async) while it waits, cover the chain where the block is long enough
-// to occupy them.  With a warp group per rank (schedule.cu) every block
-// crosses L2 once per tree edge and direction, each time behind such a chain;
-// here one edge in fifteen does.  Measured (captured calls, inputs larger
-// than L2, before and after): p = 1152 int32, m = 2^16 in 246 and 170 us,
-// m = 2^18 673 and 573; p = 288, m = 212500 244 and 140; p = 32 float32,
-// m = 2^23, b = 16 570 and 420, b = 64 850 and 456; p = 36 2x2 matrices,
-// m = 2^20 352 and 250; reduce, then broadcast at p = 288, m = 875000 in
-// 16000-element blocks 909 and 515.
+// (cp.async) while it waits, cover the chain.  With a warp group per rank
+// (schedule.cu) every block crosses L2 once per tree edge and direction, each
+// time behind such a chain; here one edge in fifteen does.  Measured (captured
+// calls, inputs larger than L2, before and after): p = 1152 int32, m = 2^16 in
+// 246 and 148 us, m = 2^18 673 and 532; p = 288, m = 212500 244 and 129; p = 32
+// float32, m = 2^23, b = 16 570 and 395, b = 64 850 and 395; p = 36 2x2
+// matrices, m = 2^20 352 and 231; reduce, then broadcast at p = 288,
+// m = 875000 in 16000-element blocks 909 and 466.
 // Not kept: 4 units per lane (fewer, longer steps; the registers for them
 // spilled, and a spilled value comes back from L2 after every acquire); a
 // warp for each direction (the two loops together no longer fitted the
@@ -225,7 +224,8 @@ struct Runner {
     }
 
     // The partial block of step t handed up: to the cell root's row, or a dual
-    // root's exchange slot.
+    // root's exchange slot.  Before the next inputs are asked for: the release
+    // would wait for them (p = 32, m = 2^23 float32, 415 and 405 us).
     __device__ __forceinline__ void hand_up(int t, const Spot& p, const T& v) const
     {
         if (p.on) U::st_keep(s->dual ? ring(s->cell == a.root0 ? 0 : 1, t) : s->y[0] + p.off, v);
@@ -249,9 +249,9 @@ struct Runner {
     // Reduce, then broadcast.  A block passes through a cell at once.
     __device__ __forceinline__ void reduce_bcast() const
     {
-        const int steps = tail ? 1 : a.col.b * a.col.waves;
+        const int steps = tail ? 1 : a.col.steps;
         const bool root = s->par_cell < 0;
-        Pos c{0, s->g};
+        Pos c(a.col, tail ? 0 : s->g);
         Spot p = note(c, 0);
         fetch(p);
 #pragma unroll 1
@@ -260,13 +260,13 @@ struct Runner {
             if (!up(t, c.j, p, v)) return;
             const Spot was = p;
             c.advance(a.col);
+            hand_up(t, was, v);
             if (t + 1 < steps) {  // the next block's inputs
                 p = note(c, t + 1);
                 fetch(p);
             }
-            hand_up(t, was, v);
         }
-        c = Pos{0, s->g};
+        c = Pos(a.col, tail ? 0 : s->g);
 #pragma unroll 1
         for (int t = 0; t < steps; t++, c.advance(a.col)) {
             p = note(c, t);
@@ -286,9 +286,9 @@ struct Runner {
     // the step.
     __device__ __forceinline__ void algorithm_1() const
     {
-        const int steps = tail ? 1 : a.col.b * a.col.waves, D = s->depth, nlev = s->nlev;
+        const int steps = tail ? 1 : a.col.steps, D = s->depth, nlev = s->nlev;
         const bool root = s->par_cell < 0;
-        Pos c{0, s->g};
+        Pos c(a.col, tail ? 0 : s->g);
         fetch(note(c, 0));
         const int last = steps - 1 + D + nlev - 1;
 #pragma unroll 1
@@ -306,8 +306,8 @@ struct Runner {
                 const Spot p = noted(t);
                 if (!up(t, c.j, p, v)) return;
                 c.advance(a.col);
-                if (t + 1 < steps) fetch(note(c, t + 1));  // the next block's inputs
                 if (!root || s->dual) hand_up(t, p, v);
+                if (t + 1 < steps) fetch(note(c, t + 1));  // the next block's inputs
                 if (s->dual) {
                     const bool lower = s->cell == a.root0;
                     if (!wait(lane == 0, ctr(a.up, lower ? a.root1 : a.root0), s->base + uint32_t(t) + 1u,

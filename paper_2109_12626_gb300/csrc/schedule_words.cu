@@ -218,9 +218,9 @@ struct Runner {
     __device__ __forceinline__ void run() const
     {
         static_assert(kLevels == 4, "the history of final blocks is three deep");
-        const int steps = tail ? 1 : a.col.b * a.col.waves, D = s->depth, nlev = s->nlev;
+        const int steps = tail ? 1 : a.col.steps, D = s->depth, nlev = s->nlev;
         const bool root = s->par_cell < 0;
-        Pos c{0, s->g}, d{0, s->g};
+        Pos c(a.col, tail ? 0 : s->g), d(a.col, tail ? 0 : s->g);
         Spot next = spot<Op, kVec>(a.col, c, lane, tail);
         fetch(next);
         T v1{}, v2{}, v3{};
@@ -399,7 +399,7 @@ int schedule_words_launch(Plan* P, cudaStream_t s)
     a.ctl = reinterpret_cast<uint32_t*>(C.d);
     a.err = P->d_err;
     const CellSlices S = cell_slices(P, C, vec);
-    a.col = Columns{P->m, P->m / P->b, P->m % P->b, P->b, S.n, S.waves, cell_tail(P, vec)};
+    a.col = Columns{P->m, P->m / P->b, P->m % P->b, P->b, S.n, S.per_block, S.steps, cell_tail(P, vec)};
     const int lines = S.n + a.col.tail;
     a.dual = reinterpret_cast<u64*>(C.d + C.off_scratch);
     a.down = a.dual + size_t(lines) * 4 * kSlot;
@@ -410,7 +410,7 @@ int schedule_words_launch(Plan* P, cudaStream_t s)
     a.ncells = C.n;
     a.root0 = C.root0;
     a.root1 = C.root1;
-    a.used = P->b * S.waves + 1;
+    a.used = S.steps + 1;
     a.skip_rank = P->skip_rank;
     return cell_launch(words_kernel_for(P->dtype, vec), &a, int64_t(C.n) * lines, kWarps, 0, s);
 }
