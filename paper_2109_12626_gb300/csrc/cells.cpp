@@ -133,7 +133,7 @@ void make_cells(const Plan* P, int max_ranks, int max_levels, CellPlan* C, std::
         c.par_cell = h.par_cell;
         c.par_rank = h.par_rank;
         c.nlev = h.nlev;
-        unsigned again = h.nlev > 1 ? 1u << (c.n - 1) : 0u;  // positions whose finals are read again
+        unsigned again = 0;  // positions whose final blocks child cells read
         for (int t = 0; t < c.n; t++) {
             const int i = h.ranks[t], c0 = P->child0[i], c1 = P->child1[i];
             const bool in = c0 >= 0 && !top[c0];

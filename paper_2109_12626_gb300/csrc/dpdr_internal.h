@@ -71,7 +71,7 @@ struct CellDesc {
     int nlev;                  // levels
     int next;                  // nodes whose two children are roots of other cells
     int down, par_down;        // number among the cells with next > 0, the parent cell's
-    int reread;                // bit t: the final blocks of position lev_k[t] are read again
+    int reread;                // bit t: child cells read the final blocks of position lev_k[t]
     int rank[kCellRanks];      // post-order, the root last
     int node_par[kCellRanks];  // parent rank inside the cell, -1 at the root
     int tape[kCellRanks];      // bits 0-1 children in the cell, 2 child_1 of its parent,

@@ -47,10 +47,10 @@ struct FusedArgs {
     int r0, r1;
     int dual;               // 1: y = v(r0) (.) v(r1); 0: one tree, y = v(p-1)
     int64_t nvec;           // 16-byte units, or (quad) units of four single elements
-    int quad;               // rows are not all 16-byte aligned: QuadUnit instead of VecUnit
     int64_t nscalar;        // single elements after the vector units
     int64_t scalar_base;    // element index of the first single element
     int lg_wu;              // tile: log2 of vector units per row
+    int quad;               // rows are not all 16-byte aligned: QuadUnit instead of VecUnit
     int64_t vec_tiles;      // tile: number of vector tiles
     // split layout
     const int2* seg;        // [nseg] (first rank, root rank) of each subtree

@@ -222,20 +222,30 @@ __device__ __forceinline__ int give_up(const uint32_t* ctl, uint32_t epoch, uint
 }
 
 // Waits until the counter of every lane with `mine` reaches its target; rank
-// and step name the lane's exchange in an error record.  `never`: a lane
-// whose partner is silent.  False when a wait of the call expired.
+// and step name the lane's exchange in an error record.  `seen`: the value
+// that the lane read last from this counter (counters only grow, so one that
+// was already far enough is not read again).  `never`: a lane whose partner
+// is silent.  False when a wait of the call expired.
 __device__ __forceinline__ bool wait_counters(uint32_t* ctl, uint32_t* err, int64_t wait_ns,
                                               uint32_t epoch, const uint32_t* c, uint32_t target,
-                                              bool mine, bool never, int rank, int j, int step)
+                                              uint32_t& seen, bool mine, bool never, int rank, int j,
+                                              int step)
 {
     const int lane = int(threadIdx.x) & 31;
-    bool pend = never || (mine && int32_t(sched::ld_acquire(c) - target) < 0);
+    bool pend = never || (mine && int32_t(seen - target) < 0);
+    if (pend && !never) {
+        seen = sched::ld_acquire(c);
+        pend = int32_t(seen - target) < 0;
+    }
     unsigned who = __ballot_sync(kAll, pend);
     if (who) {
         const uint64_t t0 = sched::now_ns();
         unsigned polls = 0, sleep = 0;
         while (true) {
-            if (pend && !never) pend = int32_t(sched::ld_acquire(c) - target) < 0;
+            if (pend && !never) {
+                seen = sched::ld_acquire(c);
+                pend = int32_t(seen - target) < 0;
+            }
             who = __ballot_sync(kAll, pend);
             if (!who) break;
             if ((polls & 15) == 15) {

@@ -21,8 +21,8 @@ int schedule_walk_prepare(Plan* P)
     CellPlan& C = P->walk;
     C.ready = false;
     // Cells of at most 16 ranks, and of up to 20 where that takes a whole tree
-    // (p = 36: two cells of 18 ranks, m = 2^20 2x2 matrices in 231 against
-    // 329 us with six; with larger trees 20 ranks make the longest walk
+    // (p = 36: two cells of 18 ranks; 2x2 matrices, m = 2^20, took 1.3 times
+    // as long with six cells; with larger trees 20 ranks make the longest walk
     // longer: p = 1152, m = 2^16 int32 15 % slower).
     const int tree = P->r0 >= 0 ? P->p - P->p / 2 : P->p;
     std::vector<CellDesc> desc;

@@ -3,49 +3,64 @@
 // kWalkRanks ranks (dpdr_allreduce_schedule and dpdr_allreduce_reduce_bcast
 // where every schedule option is automatic; schedule_cells.cuh).
 //
-// The schedule is Algorithm 1's, round by round: in round j every rank takes
-// its children's partial blocks j, forms Y[j] = t1 (.) (t0 (.) x_i) and hands
-// it to its parent (the dual roots exchange theirs), then receives final
-// block j - d_i, which its parent holds since round j - 1.
+// The schedule is Algorithm 1's: in round j every rank takes its children's
+// partial blocks j, forms Y[j] = t1 (.) (t0 (.) x_i) and hands it to its
+// parent (the dual roots exchange theirs); a rank at depth d receives final
+// block j - d.  A cell whose root is at depth D does this for all its ranks at
+// once: in step t the partial block t goes up through them, and then the final
+// block t - D goes down to all of them.  So a rank l levels below the cell's
+// root has a final block up to l rounds before the schedule asks for it, and a
+// child cell, which takes it from there l + 1 rounds later, seldom waits.
 //
 // What bounds it: a step of a warp (32 units of all its ranks, 8 KB in and
-// 8 KB out for 16 ranks) is a chain of about 6 us -- the children's counters
-// and partial blocks, the fold, a release fence, the parent's counter and
-// final block, the stores, another fence -- and device memory.  24 warps per
-// SM, each with its next step's inputs on their way into shared memory
-// (cp.async) while it waits, cover the chain.  With a warp group per rank
-// (schedule.cu) every block crosses L2 once per tree edge and direction, each
-// time behind such a chain; here one edge in fifteen does.  Measured (captured
-// calls, inputs larger than L2, before and after): p = 1152 int32, m = 2^16 in
-// 246 and 148 us, m = 2^18 673 and 532; p = 288, m = 212500 244 and 129; p = 32
-// float32, m = 2^23, b = 16 570 and 395, b = 64 850 and 395; p = 36 2x2
-// matrices, m = 2^20 352 and 231; reduce, then broadcast at p = 288,
-// m = 875000 in 16000-element blocks 909 and 466.
+// 8 KB out for 16 ranks) is a chain of about 8 us -- the children's counters
+// and partial blocks, the fold, a release fence, the parent's final block, the
+// stores, another fence -- and device memory.  24 warps per SM, each with its
+// next step's inputs on their way into shared memory (cp.async) while it
+// waits, cover most of the chain; the warps of cells with child cells have the
+// longest one.  With a warp group per rank (schedule.cu) every block crosses
+// L2 once per tree edge and direction, each time behind such a chain; here one
+// edge in fifteen does.  Measured (captured calls, inputs larger than L2,
+// before and after; copying the same rows in the same pieces takes 102, 385,
+// 340 and 322 us for the first, second, fourth and sixth): p = 1152 int32,
+// m = 2^16 in 246 and 126 us, m = 2^18 673 and 476; p = 288, m = 212500 244
+// and 113; p = 32 float32, m = 2^23, b = 16 570 and 365; p = 36 2x2 matrices,
+// m = 2^20 352 and 215; reduce, then broadcast at p = 288, m = 875000 in
+// 16000-element blocks 909 and 425.
+// Of that: final blocks to all ranks of a cell at once, not level by level,
+// p = 1152 151 to 136 us and p = 32 395 to 361; the children's values through
+// free shared-memory slots (stage) 133 to 130 and, reduced then broadcast, 457
+// to 424; one fence for both counters of a step 130 to 126 and, m = 2^18, 496
+// to 476; the parent's final block read ahead of the fold, m = 2^18, 521 to 507.
 // Not kept: 4 units per lane (fewer, longer steps; the registers for them
 // spilled, and a spilled value comes back from L2 after every acquire); a
 // warp for each direction (the two loops together no longer fitted the
 // instruction cache: 1.5 to 2.5 times as long); inputs in registers instead
-// of shared memory, 32 warps of 64 registers (p = 1152 16 % faster, blocks
-// that do not fill the GPU 20 % slower).
+// of shared memory; bulk copies of the inputs, one lane per row (8 % slower at
+// p = 32), and of the outputs (their buffers cost a quarter of the warps); the
+// counter ahead of the rows that no other cell reads (a second pass over the
+// rows, 4 % slower).
 //
 // Exchanges between cells: the cell root's partial block goes to its y row
 // (a dual root's to an exchange slot) and a release store of the cell's up
 // counter publishes it; a final block is read from the parent rank's y row
-// once the parent cell's done counter says that it finished round j - 1.
-// Counters never repeat (finish_call), so a call is one kernel and a
-// captured graph replays.
+// once the parent cell's done counter says that it finished the step that put
+// it there.  Counters never repeat (finish_call), so a call is one kernel and
+// a captured graph replays.
 //
-// Order and reuse.  A cell waits in round j for its children's partial blocks
-// j, which they publish before they wait for anything later than round
-// j - 1, for the dual root's partial j, published before the wait, and for
-// its parent's round j - 1: with all CTAs resident (cooperative launch)
-// nothing deadlocks.  The final block j overwrites partial block j in the
-// cell root's y row only after the parent has read it, and an exchange slot
-// of parity j & 1 is written again in round j + 2, after the dual's partial
-// j + 1 has shown that it finished round j.  In place (y_i == x_i) every lane
-// reads x_i of a block before it writes any y_i of it.  Every wait is bounded
-// in time; an expired wait records {rank, round, step}, marks the call's
-// epoch aborted and every other wait of the call gives up.
+// Order and reuse.  A cell waits in step t for its children's partial blocks
+// t, which they publish before they wait for any final block of their own step
+// t; for the dual root's partial t, published before the wait; and for a step
+// before t of its parent's cell, whose partial blocks it published in earlier
+// steps (a partial block is published together with the step's end only where
+// the parent's block is there already): with all CTAs resident (cooperative
+// launch) nothing deadlocks.  The final block overwrites the partial block in
+// the cell root's y row only after the parent, which holds it, has read that,
+// and an exchange slot of parity t & 1 is written again in step t + 2, after
+// the dual's partial t + 1 has shown that it finished step t.  In place
+// (y_i == x_i) every lane reads x_i of a block before it writes any y_i of it.
+// Every wait is bounded in time; an expired wait records {rank, round, step},
+// marks the call's epoch aborted and every other wait of the call gives up.
 #pragma once
 
 #include "schedule_cells.cuh"
@@ -72,7 +87,7 @@ struct WalkArgs {
     const CellDesc* cells;
     uint32_t* ctl;
     uint32_t* up;        // [cells][slices] lines: partial blocks published
-    uint32_t* done;      // the same: rounds finished
+    uint32_t* done;      // the same: steps finished
     int64_t ctr_words;   // of both
     uint32_t* err;
     char* ring;          // [2 sides][2][slices] exchange slots of 512 bytes
@@ -90,11 +105,12 @@ struct WarpInfo {        // one per warp, in shared memory
     const char* ext[2 * kExt];  // y rows of the child cells' roots
     const char* par;            // y row of the parent rank
     uint8_t tape[kRanks];       // CellDesc::tape
-    int lev_off[kLevels + 1];
     int ext_k[kExt];
     int ext_cell[2 * kExt];
     int ext_node[kExt];         // the nodes' ranks
-    int n, next, nlev, depth, root, par_cell;
+    int n, next, depth, root, par_cell;
+    int lag;                    // levels from the parent cell's root
+    int staged;                 // nodes whose children's values fit the slots
     unsigned reread;            // bit t: row y[t] is read again
     int cell, g;                // this warp's cell and column slice
     uint32_t epoch, base;       // of the call: abort mark, counter base
@@ -140,10 +156,18 @@ struct Runner {
     {
         return t + (int64_t(c) * (a.col.nslices + a.col.tail) + s->g) * kCtr;
     }
-    __device__ __forceinline__ bool wait(bool mine, const uint32_t* c, uint32_t target, bool never,
-                                         int rank, int j, int step) const
+    __device__ __forceinline__ bool wait(bool mine, const uint32_t* c, uint32_t target, uint32_t& seen,
+                                         bool never, int rank, int j, int step) const
     {
-        return wait_counters(a.ctl, a.err, a.wait_ns, s->epoch, c, target, mine, never, rank, j, step);
+        return wait_counters(a.ctl, a.err, a.wait_ns, s->epoch, c, target, seen, mine, never, rank, j, step);
+    }
+    // Whether the counter has reached its target: read once, no wait.
+    __device__ __forceinline__ bool reached(const uint32_t* c, uint32_t target, uint32_t& seen) const
+    {
+        if (lane == 0 && int32_t(seen - target) < 0) seen = sched::ld_acquire(c);
+        const bool ok = __shfl_sync(kAll, int(int32_t(seen - target) >= 0), 0) != 0;
+        __syncwarp();
+        return ok;
     }
     __device__ __forceinline__ void publish(uint32_t* t, uint32_t v) const
     {
@@ -188,22 +212,28 @@ struct Runner {
         return acc;
     }
 
-    // Steps child_0 and child_1 of step t (round j of its wave), the inputs
-    // being on their way into the slots: v becomes the cell's partial block.
-    // Returns false when a wait expired.
-    __device__ __forceinline__ bool up(int t, int j, const Spot& p, T& v) const
+    // Steps child_0 and child_1 of step t (of block j), the inputs being on
+    // their way into the slots: v becomes the cell's partial block.  Returns
+    // false when a wait expired.
+    __device__ __forceinline__ bool up(int t, int j, const Spot& p, uint32_t& seen, T& v) const
     {
         const int next = s->next;
         if (next || s->stuck >= 0) {
             const bool mine = lane < 2 * next, never = s->stuck >= 0 && lane == 31;
-            if (!wait(mine, ctr(a.up, mine ? s->ext_cell[lane] : 0), s->base + uint32_t(t) + 1u, never,
+            if (!wait(mine, ctr(a.up, mine ? s->ext_cell[lane] : 0), s->base + uint32_t(t) + 1u, seen, never,
                       never ? s->stuck : mine ? s->ext_node[lane >> 1] : 0, j,
                       never ? s->stuck_step : lane & 1))
                 return false;
         }
+        // the first nodes' values by way of the slots that the cell's ranks
+        // leave free, the others' through registers, kNodes at a time
+        const int staged = kVec ? s->staged : 0, n = s->n;
+#pragma unroll 2
+        for (int h = 0; h < 2 * staged; h++)
+            if (p.on) U::copy(slot + (n + h) * 32, s->ext[h] + p.off);
         bool landed = false;
 #pragma unroll 1
-        for (int q0 = 0; q0 < next; q0 += kNodes) {
+        for (int q0 = staged; q0 < next; q0 += kNodes) {
             T e[2 * kNodes];
 #pragma unroll
             for (int h = 0; h < 2 * kNodes; h++)
@@ -219,17 +249,23 @@ struct Runner {
                 }
         }
         if (!landed) cp_async_wait_all();
+#pragma unroll 1
+        for (int q = 0; q < staged; q++) {
+            const int k = s->ext_k[q];
+            at(k) = U::op(at(n + 2 * q + 1), U::op(at(n + 2 * q), at(k)));
+        }
         v = fold();
         return true;
     }
 
     // The partial block of step t handed up: to the cell root's row, or a dual
-    // root's exchange slot.  Before the next inputs are asked for: the release
-    // would wait for them (p = 32, m = 2^23 float32, 415 and 405 us).
-    __device__ __forceinline__ void hand_up(int t, const Spot& p, const T& v) const
+    // root's exchange slot, and published (now) or left to the step's end.
+    // Before the next inputs are asked for: the release would wait for them
+    // (p = 32, m = 2^23 float32, 415 and 405 us).
+    __device__ __forceinline__ void hand_up(int t, const Spot& p, const T& v, bool now) const
     {
         if (p.on) U::st_keep(s->dual ? ring(s->cell == a.root0 ? 0 : 1, t) : s->y[0] + p.off, v);
-        publish(a.up, s->base + uint32_t(t) + 1u);
+        if (now) publish(a.up, s->base + uint32_t(t) + 1u);
     }
 
     // v: a final block's unit, into the rows y[t0 .. t1)
@@ -251,16 +287,17 @@ struct Runner {
     {
         const int steps = tail ? 1 : a.col.steps;
         const bool root = s->par_cell < 0;
+        uint32_t up_seen = s->base, seen = s->base;  // read last from the children's, the parent's counter
         Pos c(a.col, tail ? 0 : s->g);
         Spot p = note(c, 0);
         fetch(p);
 #pragma unroll 1
         for (int t = 0; t < steps; t++) {
             T v;
-            if (!up(t, c.j, p, v)) return;
+            if (!up(t, c.j, p, up_seen, v)) return;
             const Spot was = p;
             c.advance(a.col);
-            hand_up(t, was, v);
+            hand_up(t, was, v, true);
             if (t + 1 < steps) {  // the next block's inputs
                 p = note(c, t + 1);
                 fetch(p);
@@ -270,8 +307,8 @@ struct Runner {
 #pragma unroll 1
         for (int t = 0; t < steps; t++, c.advance(a.col)) {
             p = note(c, t);
-            if (!root && !wait(lane == 0, ctr(a.done, s->par_cell), s->base + uint32_t(t) + 1u, false,
-                               s->root, c.j, 3))
+            if (!root && !wait(lane == 0, ctr(a.done, s->par_cell), s->base + uint32_t(t) + 1u,
+                               seen, false, s->root, c.j, 3))
                 return;
             T v{};
             if (p.on) v = U::ld((root ? s->y[0] : s->par) + p.off);  // a root holds the block
@@ -280,38 +317,43 @@ struct Runner {
         }
     }
 
-    // Algorithm 1.  A final block that reaches the cell's root in step t
-    // reaches the ranks l levels below it in step t + l, from the cell root's
-    // row, which holds it since: those loads are under way from the start of
-    // the step.
+    // Algorithm 1, a step at a time.
     __device__ __forceinline__ void algorithm_1() const
     {
-        const int steps = tail ? 1 : a.col.steps, D = s->depth, nlev = s->nlev;
+        const int steps = tail ? 1 : a.col.steps, D = s->depth;
         const bool root = s->par_cell < 0;
+        // read last from the children's counters, the dual's or the parent's
+        uint32_t up_seen = s->base, seen = s->base;
         Pos c(a.col, tail ? 0 : s->g);
         fetch(note(c, 0));
-        const int last = steps - 1 + D + nlev - 1;
+        const int last = steps - 1 + D;
 #pragma unroll 1
         for (int t = 0; t <= last; t++) {
-            const int f = t - D;  // the step whose block is final at the cell's root now
-            T h[kLevels - 1];
-#pragma unroll
-            for (int l = 1; l < kLevels; l++)
-                if (l < nlev && f - l >= 0 && f - l < steps) {
-                    const Spot q = noted(f - l);
-                    if (q.on) h[l - 1] = U::ld(s->y[0] + q.off);
+            const int f = t - D;  // the step whose block is final in this cell now
+            // the parent's cell put it there in step t - lag: read ahead of the
+            // fold where that is over
+            const uint32_t final_at = s->base + uint32_t(t - s->lag) + 1u;
+            T v{}, w{};
+            bool held = false;
+            if (f >= 0 && !root) {
+                held = reached(ctr(a.done, s->par_cell), final_at, seen);
+                if (held) {
+                    const Spot p = noted(f);
+                    if (p.on) w = U::ld(s->par + p.off);
                 }
-            T v{};
+            }
+            // one fence for both counters where nothing of this step waits
+            const bool join = held && t < steps && s->next;
             if (t < steps) {
                 const Spot p = noted(t);
-                if (!up(t, c.j, p, v)) return;
+                if (!up(t, c.j, p, up_seen, v)) return;
                 c.advance(a.col);
-                if (!root || s->dual) hand_up(t, p, v);
+                if (!root || s->dual) hand_up(t, p, v, !join);
                 if (t + 1 < steps) fetch(note(c, t + 1));  // the next block's inputs
                 if (s->dual) {
                     const bool lower = s->cell == a.root0;
                     if (!wait(lane == 0, ctr(a.up, lower ? a.root1 : a.root0), s->base + uint32_t(t) + 1u,
-                              false, s->root, c.j, 2))
+                              seen, false, s->root, c.j, 2))
                         return;
                     if (p.on) {
                         const T o = U::ld(ring(lower ? 1 : 0, t));
@@ -320,20 +362,25 @@ struct Runner {
                 }
             }
             if (f < 0) continue;
-#pragma unroll
-            for (int l = 1; l < kLevels; l++)
-                if (l < nlev && f - l >= 0 && f - l < steps)
-                    put(noted(f - l), h[l - 1], s->lev_off[l], s->lev_off[l + 1]);
-            if (f < steps) {
-                const Spot p = noted(f);
-                if (!root) {
-                    if (!wait(lane == 0, ctr(a.done, s->par_cell), s->base + uint32_t(t), false, s->root, t, 3))
-                        return;
-                    if (p.on) v = U::ld(s->par + p.off);
+            const Spot p = noted(f);
+            if (!root) {
+                if (!held) {
+                    if (!wait(lane == 0, ctr(a.done, s->par_cell), final_at, seen, false, s->root, t, 3)) return;
+                    if (p.on) w = U::ld(s->par + p.off);
                 }
-                put(p, v, 0, 1);
+                v = w;
             }
-            if (s->next) publish(a.done, s->base + uint32_t(t) + 1u);
+            put(p, v, 0, s->n);
+            if (join) {
+                __syncwarp();
+                if (lane == 0 && !s->mute) {
+                    __threadfence();
+                    sched::st_relaxed(ctr(a.up, s->cell), s->base + uint32_t(t) + 1u);
+                    sched::st_relaxed(ctr(a.done, s->cell), s->base + uint32_t(t) + 1u);
+                }
+            } else if (s->next) {
+                publish(a.done, s->base + uint32_t(t) + 1u);
+            }
         }
     }
 };
@@ -368,15 +415,15 @@ __global__ void __launch_bounds__(kWarps * 32, kCtas) walk_kernel(const __grid_c
             s->ext_k[lane] = __ldg(c->ext_k + lane);
             s->ext_node[lane] = __ldg(c->rank + __ldg(c->ext_k + lane));
         }
-        if (lane <= kLevels) s->lev_off[lane] = __ldg(c->lev_off + lane);
         if (lane == 31) {
             const int par = __ldg(&c->par_rank);
             s->n = n;
             s->next = next;
-            s->nlev = __ldg(&c->nlev);
+            s->staged = min(next, (a.ranks - n) / 2);
             s->depth = __ldg(&c->depth);
             s->root = __ldg(&c->root);
             s->par_cell = __ldg(&c->par_cell);
+            s->lag = s->par_cell < 0 ? 0 : s->depth - __ldg(&a.cells[s->par_cell].depth);
             s->reread = unsigned(__ldg(&c->reread));
             if (par >= 0) s->par = sched::rank_out(a.y, par);
             s->cell = cell;

@@ -179,10 +179,12 @@ struct Runner {
     {
         const int next = s->next;
         const uint32_t flag = s->base + uint32_t(t) + 1u;
-        if (s->stuck >= 0)  // the silent rank of the fault injection: wait in vain
-            if (!wait_counters(a.ctl, a.err, a.wait_ns, s->epoch, a.ctl, 0, false, lane == 0, s->stuck, j,
-                               s->stuck_step))
+        if (s->stuck >= 0) {  // the silent rank of the fault injection: wait in vain
+            uint32_t seen = 0;
+            if (!wait_counters(a.ctl, a.err, a.wait_ns, s->epoch, a.ctl, 0, seen, false, lane == 0,
+                               s->stuck, j, s->stuck_step))
                 return false;
+        }
         bool landed = false;
 #pragma unroll 1
         for (int q0 = 0; q0 < next; q0 += kNodes) {

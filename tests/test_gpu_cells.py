@@ -5,7 +5,8 @@ both entry points and both topologies.
 
 Sizes are the edges of the cell layout: one cell, cells of one rank, the
 first cut edges (p = 15, 16, 36), ragged last levels; slices of one unit, of
-32, partly filled, several to a warp, of two blocks in a step; blocks that start and end inside a
+32, partly filled, several to a warp, of two blocks in a step; blocks that
+start and end inside a
 16-byte unit or lie within one, rows with a ragged tail."""
 import numpy as np
 import pytest
