@@ -340,6 +340,7 @@ int fused_launch_cols(Plan* P, const char* const* dx, char* const* dy, int64_t m
     a.tree_s = T.s;
     a.tree_slots = T.slots;
     a.tree_width = T.width;
+    a.overlap = dx == P->d_x && !force_mode;  // device buffers, no chunks between copies
     a.tree_tiles = T.width ? (a.nvec + T.width - 1) / T.width : 0;
 
     switch (mode) {

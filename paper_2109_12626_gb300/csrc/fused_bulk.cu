@@ -105,6 +105,7 @@ template <class Op>
 __global__ void __launch_bounds__(kBulkThreads, 2)
 fused_bulk_kernel(FusedArgs a)
 {
+    wait_previous();
     extern __shared__ __align__(128) uint4 smem[];
     char* base = reinterpret_cast<char*>(smem);
     char* ring = base;                                            // [S][tile]
@@ -219,8 +220,7 @@ struct Bulk {
         const int64_t tail = (a.nvec - a.bulk_tiles * (kBulkTile / 16)) + a.nscalar;
         int64_t grid = std::min<int64_t>(a.bulk_tiles, resident);
         grid = std::max<int64_t>(grid, std::min<int64_t>(resident, (tail + kBulkConsumers - 1) / kBulkConsumers));
-        fused_bulk_kernel<Op><<<unsigned(std::max<int64_t>(grid, 1)), kBulkThreads, smem, s>>>(a);
-        return launched();
+        return launch_kernel(&fused_bulk_kernel<Op>, dim3(unsigned(std::max<int64_t>(grid, 1))), kBulkThreads, smem, s, a);
     }
 };
 

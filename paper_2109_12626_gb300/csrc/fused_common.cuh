@@ -71,6 +71,7 @@ struct FusedArgs {
     int tree_nseg, tree_nlev, tree_r0, tree_r1, tree_s, tree_slots;
     int64_t tree_tiles;     // CTAs of tree_width vector units
     int tree_width;         // kTreeUnitsNarrow or kTreeUnitsWide
+    int overlap;            // launch: set up while the kernel before drains
 };
 
 template <class Op>
@@ -278,11 +279,36 @@ int dispatch(Plan* P, FusedArgs a, cudaStream_t s)
     }
 }
 
-inline int launched()
+// The fused kernels are launched with programmatic stream serialisation: a
+// kernel is set up while the one before it in the stream drains, and its
+// threads wait here, before they touch any memory, until that one is complete
+// and its writes are visible.  So calls are ordered as ever, and so is what
+// follows in the stream; what goes is the gap between two kernels (back to
+// back, p = 7, m = 1000 int32 in 4.1 and 2.7 us; p = 36, m = 2^16 2x2 matrices
+// 16.4 and 14.5; p = 1152 int32, m = 1024 10.3 and 8.9, and m = 2^16, two
+// kernels of the split layout, 113 and 107).
+// No kernel asks for the next one to start early, so a CTA never
+// waits here in a place that a running kernel needs.  Calls on host memory
+// are launched the plain way: they gain nothing, and back to back their reads
+// and writes share the link less evenly (p = 36, m = 2^16 2x2 matrices 242
+// against 230 us).
+__device__ __forceinline__ void wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+inline int launch_kernel(void (*kernel)(FusedArgs), dim3 grid, int threads, size_t smem, cudaStream_t s,
+                         const FusedArgs& a)
 {
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return cuda_fail(e, "fused kernel launch");
-    return DPDR_OK;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(unsigned(threads));
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = a.overlap ? 1 : 0;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, a);
+    return e == cudaSuccess ? DPDR_OK : cuda_fail(e, "fused kernel launch");
 }
 
 }  // namespace fused

@@ -75,6 +75,7 @@ template <class Op, class V>
 __global__ void __launch_bounds__(kStreamThreads, 4)
 fused_split_reduce_kernel(FusedArgs a)
 {
+    wait_previous();
     extern __shared__ uint4 smem[];
     const int64_t u = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     if (u < a.nvec) {
@@ -90,6 +91,7 @@ template <class Op, class V>
 __global__ void __launch_bounds__(kStreamThreads, 4)
 fused_split_finish_kernel(FusedArgs a)
 {
+    wait_previous();
     extern __shared__ uint4 smem[];
     const int64_t u = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     if (u < a.nvec) {
@@ -123,11 +125,11 @@ struct Split {
                     return rc;
             }
             const int groups = (P->p + a.group - 1) / a.group;
-            fused_split_reduce_kernel<Op, V>
-                <<<dim3(unsigned(blocks), unsigned(P->split_nseg)), kStreamThreads, smem, s>>>(a);
-            fused_split_finish_kernel<Op, V>
-                <<<dim3(unsigned(blocks), unsigned(groups)), kStreamThreads, smem, s>>>(a);
-            return launched();
+            if (int rc = launch_kernel(&fused_split_reduce_kernel<Op, V>,
+                                dim3(unsigned(blocks), unsigned(P->split_nseg)), kStreamThreads, smem, s, a))
+                return rc;
+            return launch_kernel(&fused_split_finish_kernel<Op, V>, dim3(unsigned(blocks), unsigned(groups)),
+                          kStreamThreads, smem, s, a);
         });
     }
 };

@@ -21,6 +21,7 @@ template <class Op, class V>
 __global__ void __launch_bounds__(kStreamThreads, 4)
 fused_stream_kernel(FusedArgs a)
 {
+    wait_previous();
     extern __shared__ uint4 smem[];
     const int64_t u = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     if (u < a.nvec) {
@@ -90,6 +91,7 @@ template <class Op, class V>
 __global__ void __launch_bounds__(kStreamThreads, 4)
 fused_stream_pair_kernel(FusedArgs a)
 {
+    wait_previous();
     extern __shared__ uint4 smem[];
     const int lane = threadIdx.x & 31, h = lane >> 4;
     const int64_t c = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) / 32 * 16 + (lane & 15);
@@ -117,15 +119,10 @@ struct Stream {
         if (blocks > 0x7fffffff) return fail(DPDR_ERR_INVALID, "m too large");
         return with_unit<Op, kQuadStream>(a, [&](auto unit) {
             using V = decltype(unit);
-            const void* kern = pairs ? reinterpret_cast<const void*>(&fused_stream_pair_kernel<Op, V>)
-                                     : reinterpret_cast<const void*>(&fused_stream_kernel<Op, V>);
+            void (*const kern)(FusedArgs) = pairs ? &fused_stream_pair_kernel<Op, V> : &fused_stream_kernel<Op, V>;
             int* const granted = &P->smem_attr[(pairs ? 6 : 0) + (a.quad ? kQuadAttr : 0)];
-            if (int rc = grant_smem(kern, smem, granted, "fused stream attribute")) return rc;
-            if (pairs)
-                fused_stream_pair_kernel<Op, V><<<unsigned(blocks), kStreamThreads, smem, s>>>(a);
-            else
-                fused_stream_kernel<Op, V><<<unsigned(blocks), kStreamThreads, smem, s>>>(a);
-            return launched();
+            if (int rc = grant_smem(reinterpret_cast<const void*>(kern), smem, granted, "fused stream attribute")) return rc;
+            return launch_kernel(kern, dim3(unsigned(blocks)), kStreamThreads, smem, s, a);
         });
     }
 };

@@ -103,6 +103,7 @@ template <class Op, class V>
 __global__ void __launch_bounds__(kTileThreads)
 fused_tile_kernel(FusedArgs a)
 {
+    wait_previous();
     extern __shared__ uint4 smem[];
     const int64_t t = blockIdx.x;
     // a narrow last tile (small m) is packed with a row stride of its own
@@ -136,8 +137,7 @@ struct Tile {
             if (int rc = grant_smem(reinterpret_cast<const void*>(&fused_tile_kernel<Op, V>), smem,
                                     &P->smem_attr[1 + (a.quad ? kQuadAttr : 0)], "fused tile attribute"))
                 return rc;
-            fused_tile_kernel<Op, V><<<unsigned(blocks), kTileThreads, smem, s>>>(a);
-            return launched();
+            return launch_kernel(&fused_tile_kernel<Op, V>, dim3(unsigned(blocks)), kTileThreads, smem, s, a);
         });
     }
 };

@@ -117,6 +117,7 @@ template <class Op, class V, int W>
 __global__ void __launch_bounds__(kTreeThreads, 2)
 fused_tree_kernel(FusedArgs a)
 {
+    wait_previous();
     extern __shared__ uint4 smem[];
     const int tid = threadIdx.x;
     if (blockIdx.x < a.tree_tiles) {
@@ -149,8 +150,7 @@ struct Tree {
             const void* kern = reinterpret_cast<const void*>(&fused_tree_kernel<Op, V, W>);
             int* const granted = &P->smem_attr[(wide ? 5 : 4) + (a.quad ? kQuadAttr : 0)];
             if (int rc = grant_smem(kern, smem, granted, "fused tree attribute")) return rc;
-            fused_tree_kernel<Op, V, W><<<unsigned(blocks), kTreeThreads, smem, s>>>(a);
-            return launched();
+            return launch_kernel(&fused_tree_kernel<Op, V, W>, dim3(unsigned(blocks)), kTreeThreads, smem, s, a);
         };
         constexpr int N = kTreeUnitsNarrow, W = kTreeUnitsWide;
         return wide ? with_unit<Op, W>(a, [&](auto u) { return launch(u, std::integral_constant<int, W>()); })
