@@ -394,24 +394,25 @@ __global__ void __launch_bounds__(kWarps * 32, kCtas) walk_kernel(const __grid_c
     __shared__ WarpInfo info[kWarps];
     const int lane = int(threadIdx.x) & 31, w = int(threadIdx.x >> 5);
     const int64_t gw = int64_t(blockIdx.x) * kWarps + w;
-    const uint32_t epoch = *reinterpret_cast<volatile const uint32_t*>(a.ctl);
-    const uint32_t base = *reinterpret_cast<volatile const uint32_t*>(a.ctl + 3);
+    Call call = ask_call(a.ctl);
     const int lines = a.col.nslices + a.col.tail;  // the tail slice comes last
-    if (gw < int64_t(a.ncells) * lines) {
-        WarpInfo* const s = &info[w];
-        const int cell = int(gw / lines), g = int(gw % lines);
+    const bool here = gw < int64_t(a.ncells) * lines;
+    const int cell = int(gw / lines), g = int(gw % lines);
+    WarpInfo* const s = &info[w];
+    if (here) {
         const CellDesc* c = a.cells + cell;
         const int n = __ldg(&c->n), next = __ldg(&c->next);
-        if (lane < n) {
+        // past its ranks and nodes a descriptor holds zeros: no need to wait for n
+        if (lane < kRanks) {
             s->x[lane] = sched::rank_in(a.x, __ldg(c->rank + lane));
             s->y[lane] = sched::rank_out(a.y, __ldg(c->rank + __ldg(c->lev_k + lane)));
             s->tape[lane] = uint8_t(__ldg(c->tape + lane));
         }
-        if (lane < 2 * next) {
+        if (lane < 2 * kExt) {
             s->ext[lane] = sched::rank_out(a.y, __ldg(c->ext_rank + lane));
             s->ext_cell[lane] = __ldg(c->ext_cell + lane);
         }
-        if (lane < next) {
+        if (lane < kExt) {
             s->ext_k[lane] = __ldg(c->ext_k + lane);
             s->ext_node[lane] = __ldg(c->rank + __ldg(c->ext_k + lane));
         }
@@ -428,8 +429,6 @@ __global__ void __launch_bounds__(kWarps * 32, kCtas) walk_kernel(const __grid_c
             if (par >= 0) s->par = sched::rank_out(a.y, par);
             s->cell = cell;
             s->g = g;
-            s->epoch = epoch;
-            s->base = base;
             s->dual = a.root0 >= 0 && par < 0;
             s->mute = a.skip_rank >= 0 && s->root == a.skip_rank;
             s->stuck = -1;
@@ -440,6 +439,13 @@ __global__ void __launch_bounds__(kWarps * 32, kCtas) walk_kernel(const __grid_c
                         s->stuck = __ldg(c->node_par + k);
                         s->stuck_step = (__ldg(c->tape + k) & 4) ? 1 : 0;
                     }
+        }
+    }
+    start_call(a.ctl, call);
+    if (here) {
+        if (lane == 0) {
+            s->epoch = call.epoch;
+            s->base = call.base;
         }
         __syncwarp();
         uint4* const slot = walk_slots + w * a.ranks * 32 + lane;
@@ -454,7 +460,7 @@ __global__ void __launch_bounds__(kWarps * 32, kCtas) walk_kernel(const __grid_c
         }
         cp_async_wait_all();
     }
-    finish_call(a.ctl, epoch, base, uint32_t(a.used), a.up, a.ctr_words);
+    finish_call(a.ctl, call, uint32_t(a.used), a.up, a.ctr_words);
 }
 
 template <bool kRB>

@@ -280,22 +280,23 @@ __global__ void __launch_bounds__(kWarps * 32, 4) words_kernel(const __grid_cons
     __shared__ WarpInfo info[kWarps];
     const int lane = int(threadIdx.x) & 31, w = int(threadIdx.x) >> 5;
     const int64_t gw = int64_t(blockIdx.x) * kWarps + w;
-    const uint32_t epoch = *reinterpret_cast<volatile const uint32_t*>(a.ctl);
-    const uint32_t base = *reinterpret_cast<volatile const uint32_t*>(a.ctl + 3);
+    Call call = ask_call(a.ctl);
     const int lines = a.col.nslices + a.col.tail;  // the tail slice comes last
-    if (gw < int64_t(a.ncells) * lines) {
-        const int cell = int(gw / lines), g = int(gw % lines);
-        WarpInfo* s = &info[w];
+    const bool here = gw < int64_t(a.ncells) * lines;
+    const int cell = int(gw / lines), g = int(gw % lines);
+    WarpInfo* const s = &info[w];
+    if (here) {
         const CellDesc* c = a.cells + cell;
         const int n = __ldg(&c->n), next = __ldg(&c->next);
-        if (lane < n) {
+        // past its ranks and nodes a descriptor holds zeros: no need to wait for n
+        if (lane < kRanks) {
             s->x[lane] = sched::rank_in(a.x, __ldg(c->rank + lane));
             s->y[lane] = sched::rank_out(a.y, __ldg(c->rank + __ldg(c->lev_k + lane)));
             reinterpret_cast<uint8_t*>(&s->tape)[lane] = uint8_t(__ldg(c->tape + lane));
         }
-        if (lane < 2 * next)
+        if (lane < 2 * kExt)
             s->up_in[lane] = a.up + (int64_t(__ldg(c->ext_cell + lane)) * lines + g) * a.up_slots * kSlot;
-        if (lane < next) s->ext_k[lane] = __ldg(c->ext_k + lane);
+        if (lane < kExt) s->ext_k[lane] = __ldg(c->ext_k + lane);
         if (lane <= kLevels) s->lev_off[lane] = __ldg(c->lev_off + lane);
         if (lane == 31) {
             const int side = cell == a.root0 ? 0 : 1;
@@ -307,8 +308,6 @@ __global__ void __launch_bounds__(kWarps * 32, 4) words_kernel(const __grid_cons
             s->par_cell = __ldg(&c->par_cell);
             s->cell = cell;
             s->g = g;
-            s->epoch = epoch;
-            s->base = base;
             s->dual = a.root0 >= 0 && s->par_cell < 0;
             s->up_out = a.up + (int64_t(cell) * lines + g) * a.up_slots * kSlot;
             s->down_in = a.down + (int64_t(__ldg(&c->par_down)) * lines + g) * kDownSlots * kSlot;
@@ -325,6 +324,13 @@ __global__ void __launch_bounds__(kWarps * 32, 4) words_kernel(const __grid_cons
                         s->stuck_step = (__ldg(c->tape + k) & 4) ? 1 : 0;
                     }
         }
+    }
+    start_call(a.ctl, call);
+    if (here) {
+        if (lane == 0) {
+            s->epoch = call.epoch;
+            s->base = call.base;
+        }
         __syncwarp();
         uint4* const slot = slots + w * kRanks * 32 + lane;
         if (kVec && Op::kEpv > 1 && g == a.col.nslices)
@@ -333,7 +339,7 @@ __global__ void __launch_bounds__(kWarps * 32, 4) words_kernel(const __grid_cons
             Runner<Op, kVec>{a, s, slot, lane, false}.run();
         cp_async_wait_all();
     }
-    finish_call(a.ctl, epoch, base, uint32_t(a.used), reinterpret_cast<uint32_t*>(a.dual), a.words);
+    finish_call(a.ctl, call, uint32_t(a.used), reinterpret_cast<uint32_t*>(a.dual), a.words);
 }
 
 template <class Op>
