@@ -56,7 +56,14 @@ KERNEL_SOURCES = {"stream": ("fused_stream.cu", "fused_common.cuh"),
                   "tree": ("fused_tree.cu", "fused_common.cuh"),
                   "schedule": ("schedule.cu", "schedule_common.cuh"),
                   "schedule_words": ("schedule_ll.cu", "schedule_common.cuh"),
-                  "reduce_bcast": ("schedule.cu", "schedule_common.cuh")}
+                  "reduce_bcast": ("schedule.cu", "schedule_common.cuh"),
+                  "schedule_walk": ("schedule_walk.cu", "schedule_walk.cuh", "schedule_cells.cuh",
+                                    "cells.cpp", "fused_common.cuh", "schedule_common.cuh"),
+                  "schedule_cell_words": ("schedule_words.cu", "schedule_cells.cuh", "cells.cpp",
+                                          "fused_common.cuh", "schedule_common.cuh"),
+                  "reduce_bcast_walk": ("schedule_walk_rb.cu", "schedule_walk.cuh",
+                                        "schedule_cells.cuh", "cells.cpp", "fused_common.cuh",
+                                        "schedule_common.cuh")}
 LAYOUTS = {1: "stream", 2: "tile", 3: "split", 4: "bulk", 5: "tree"}
 
 
@@ -785,9 +792,11 @@ def main(argv=None) -> int:
                "sample": sample}
 
     info = plan.info()
+    cells = info["sched_cells"] > 0  # every schedule option automatic: the kernels on subtree cells
     layout = (LAYOUTS[args.mode or info["auto_mode"]] if args.kernel == "fused"
-              else "reduce_bcast" if args.kernel == "reduce_bcast"
-              else ("schedule", "schedule_words")[info["sched_transport"] - 1])
+              else ("reduce_bcast", "reduce_bcast_walk")[cells] if args.kernel == "reduce_bcast"
+              else (("schedule", "schedule_walk"),
+                    ("schedule_words", "schedule_cell_words"))[info["sched_transport"] - 1][cells])
     launches_per_step = 2 if layout == "split" else 1
     line = {
         "metric": METRIC, "value": round(value, 2), "unit": "GB/s",
@@ -799,6 +808,7 @@ def main(argv=None) -> int:
                    "topology": args.topology,
                    "kernel": args.kernel, "b": info["b"],
                    "sched_layout": (None if args.kernel == "fused" else
+                                    "%d subtree cells" % info["sched_cells"] if cells else
                                     {1: "rank ranges", 2: "by work"}[info["sched_layout"]]),
                    "fused_mode": args.mode or info["auto_mode"],
                    "split_depth": info["split_depth"] if (args.mode or info["auto_mode"]) == 3 else None,

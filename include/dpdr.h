@@ -122,8 +122,9 @@ int dpdr_block_count_rule(int p, int64_t m, double kappa);
 /* Builds the trees, the block partition and the device tables for p ranks
  * of m elements of (dtype, op) on the current CUDA device, and allocates the
  * plan's device scratch (rank-pointer tables, handshake counters, the dual
- * roots' exchange slots, an error word, and the word arrays of the
- * schedule kernel's flagged-word transport when it is selected).  b is the
+ * roots' exchange slots, an error word, and the cell tables, counters and
+ * word slots of the schedule kernels on subtree cells; the word arrays of
+ * the flagged-word transport without cells when that is selected).  b is the
  * number of pipeline blocks (Algorithm 1), clamped to [1, max(m,1)].
  * b == 0 selects a block count measured for the schedule kernel on this
  * GPU: 1 when the flagged-word transport is selected (latency-bound);
@@ -272,12 +273,19 @@ int dpdr_allreduce(dpdr_plan_t plan, const void* const* x, void* const* y,
 
 /* Schedule-faithful kernel: runs Algorithm 1 for every virtual rank, rounds
  * j = 0..b+d_i, each round's exchanges with child_0, child_1 and the parent
- * or dual, as one cooperative persistent launch in which groups of warps
- * serve ranks (DPDR_OPT_SCHED_LAYOUT) and exchange pipeline blocks through
- * device memory, published either by release/acquire counters or as
- * epoch-flagged words (DPDR_OPT_SCHED_TRANSPORT); with counters, blocks
- * move between device memory and shared memory by bulk (TMA) or per-lane
- * copies (DPDR_OPT_SCHED_COPY).  Same result as dpdr_allreduce.  Two calls
+ * or dual, as one cooperative persistent launch.  The virtual ranks are
+ * gathered into subtree cells (plan info [19]): a warp runs the ranks of a
+ * cell for a column slice of every block, hands values on between them in
+ * registers and shared memory, and exchanges blocks with other cells through
+ * device memory, published either by release/acquire counters or as flagged
+ * words.  The slices of all blocks pass in order, at most two blocks' worth
+ * in a step of the kernel, and a rank inside a cell may have a final block
+ * some rounds before Algorithm 1 asks for it.  Where a schedule option is
+ * set or the cells do not fit, groups of warps serve single ranks instead
+ * (DPDR_OPT_SCHED_LAYOUT) and exchange every block through device memory
+ * (DPDR_OPT_SCHED_TRANSPORT); with counters, blocks then move between device
+ * memory and shared memory by bulk (TMA) or per-lane copies
+ * (DPDR_OPT_SCHED_COPY).  Same result as dpdr_allreduce.  Two calls
  * on one plan that overlap on the GPU (two streams) race on its scratch.  Every wait is bounded
  * (DPDR_OPT_WAIT_LIMIT_NS); an expired wait ends the kernel early and is
  * reported as DPDR_ERR_TIMEOUT by dpdr_plan_sync.  Returns
@@ -292,8 +300,8 @@ int dpdr_allreduce_schedule(dpdr_plan_t plan, const void* const* x,
  * the root, each phase moving blocks in one direction only.  Needs a plan
  * made with DPDR_TOPO_SINGLE (the complete post-order tree over all p ranks,
  * root p-1); any other plan is DPDR_ERR_INVALID.  Runs as one cooperative
- * persistent launch with the same CTA layout, handshakes, block passes and
- * bounded waits as dpdr_allreduce_schedule's counters transport: in the
+ * persistent launch with the same cells or CTA layout, handshakes, block
+ * passes and bounded waits as dpdr_allreduce_schedule with counters: in the
  * reduction every rank forms Y[j] = v(child_1) (.) (v(child_0) (.) x_i) for
  * j = 0..b-1 and publishes it to its parent; once its reduction is done it
  * receives the final blocks from its parent in order and publishes each to
