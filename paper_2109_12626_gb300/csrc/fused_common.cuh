@@ -81,6 +81,16 @@ struct VecUnit {
     {
         return ld_stream(row + u * 16);
     }
+    // Past L1, in the paired streaming and split layouts: p = 104, m = 2^18
+    // float32 38.6 and 37.6 us, p = 1152 int32, m = 2^16 107.4 and 105.6,
+    // m = 2^20 1403 and 1394, p = 4094, m = 2^17 698 and 678, never slower.
+    // In the others it is not clear: plain streaming p = 100, m = 2^20 135.7
+    // and 134.2 but p = 62, m = 1862468 147.8 and 148.3, hierarchical tile
+    // p = 1152, m = 8192 21.7 and 21.4 but p = 576, m = 8192 12.9 and 13.0.
+    __device__ __forceinline__ static T ld_wave(const char* row, int64_t u)
+    {
+        return ld_stream_past_l1(row + u * 16);
+    }
     __device__ __forceinline__ static void st(char* row, int64_t u, const T& v)
     {
         st_stream(row + u * 16, v);
@@ -126,6 +136,7 @@ struct QuadUnit {
         const char* p = row + at(u);
         return make_uint4(ld1(p), ld1(p + kStep), ld1(p + 2 * kStep), ld1(p + 3 * kStep));
     }
+    __device__ __forceinline__ static T ld_wave(const char* row, int64_t u) { return ld(row, u); }
     __device__ __forceinline__ static void st(char* row, int64_t u, const T& v)
     {
         char* p = row + at(u);
@@ -172,6 +183,7 @@ struct OneUnit {
     {
         return ld_one_stream<Op>(row + e * Op::kEsize);
     }
+    __device__ __forceinline__ static T ld_wave(const char* row, int64_t e) { return ld(row, e); }
     __device__ __forceinline__ static void st(char* row, int64_t e, const T& v)
     {
         st_one_stream<Op>(row + e * Op::kEsize, v);

@@ -26,7 +26,7 @@ __device__ __forceinline__ void split_reduce_column(const FusedArgs& a, int g, i
     const int lo = sg.x, hi = sg.y;  // inclusive; lo is a leaf unless lo == hi
     char* row = a.part + int64_t(g) * a.part_stride;
     if (lo == hi) {  // a one-leaf subtree, or a node above the cut: its input
-        U::st_keep(row, u, U::ld(rank_ptr(a.x, lo), u));
+        U::st_keep(row, u, U::ld_wave(rank_ptr(a.x, lo), u));
         return;
     }
     T acc{};  // set by rank lo, a leaf
@@ -34,7 +34,7 @@ __device__ __forceinline__ void split_reduce_column(const FusedArgs& a, int g, i
         T cur[kStreamAhead];
 #pragma unroll
         for (int k = 0; k < kStreamAhead; k++)
-            if (i0 + k <= hi) cur[k] = U::ld(rank_ptr(a.x, i0 + k), u);
+            if (i0 + k <= hi) cur[k] = U::ld_wave(rank_ptr(a.x, i0 + k), u);
 #pragma unroll
         for (int k = 0; k < kStreamAhead; k++)
             if (i0 + k <= hi) fold_step<U>(__ldg(a.tape + i0 + k), cur[k], acc, slot, stride);

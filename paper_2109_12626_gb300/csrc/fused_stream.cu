@@ -68,7 +68,7 @@ __device__ __forceinline__ void stream_half(const FusedArgs& a, int64_t u, int h
         T cur[kStreamAhead];
 #pragma unroll
         for (int k = 0; k < kStreamAhead; k++)
-            if (i0 + k >= lo && i0 + k < hi) cur[k] = U::ld(rank_ptr(a.x, i0 + k), u);
+            if (i0 + k >= lo && i0 + k < hi) cur[k] = U::ld_wave(rank_ptr(a.x, i0 + k), u);
         const unsigned long long tp =
             __ldg(reinterpret_cast<const unsigned long long*>(a.tape + i0));
 #pragma unroll

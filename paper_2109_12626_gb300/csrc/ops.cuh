@@ -106,6 +106,15 @@ __device__ __forceinline__ uint4 ld_stream(const void* p)
 {
     return __ldcs(reinterpret_cast<const uint4*>(p));
 }
+// The same without a line in L1, which is left to the rank pointers and tables.
+__device__ __forceinline__ uint4 ld_stream_past_l1(const void* p)
+{
+    uint4 v;
+    asm volatile("ld.global.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                 : "l"(p));
+    return v;
+}
 __device__ __forceinline__ void st_stream(void* p, uint4 v)
 {
     __stcs(reinterpret_cast<uint4*>(p), v);
