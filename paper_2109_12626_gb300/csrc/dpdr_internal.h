@@ -169,9 +169,11 @@ struct Plan {
 
     // dynamic shared memory already granted to the fused kernels of this
     // plan's element type (stream, tile, split, bulk, hierarchical tile of
-    // either width, paired stream; then the same on unaligned rows), so
-    // launches skip the attribute call; the limits themselves only ever rise
-    int smem_attr[14] = {48 * 1024, 48 * 1024, 48 * 1024, 48 * 1024, 48 * 1024, 48 * 1024, 48 * 1024,
+    // either width, paired stream; then the same on unaligned rows and for
+    // inputs many times L2), so launches skip the attribute call; the limits
+    // themselves only ever rise
+    int smem_attr[21] = {48 * 1024, 48 * 1024, 48 * 1024, 48 * 1024, 48 * 1024, 48 * 1024, 48 * 1024,
+                         48 * 1024, 48 * 1024, 48 * 1024, 48 * 1024, 48 * 1024, 48 * 1024, 48 * 1024,
                          48 * 1024, 48 * 1024, 48 * 1024, 48 * 1024, 48 * 1024, 48 * 1024, 48 * 1024};
 
     // split layout of the fused kernel (fused.cu): subtrees at depth split_s

@@ -158,6 +158,21 @@ int fused_auto_mode(const Plan* P)
     return P->split_ready ? 3 : 1;
 }
 
+// Inputs of which L2 holds a thirtieth at most are loaded past L1 at normal L2
+// priority (FarUnit), where few or many ranks share a column (min of 3 runs,
+// two places in memory): p = 1152, m = 2^22 float32 5405 against 5427 us, m =
+// 2^20 1476 against 1491, m = 5000000 6475 against 6518; p = 4094, m = 2^19
+// 2851 against 2875; p = 32, m = 2^27 4910 against 4914 and 4916 against 4960;
+// p = 2, m = 2^29 1427 against 1434.  Between, the streaming hints are level
+// or better (p = 64, m = 3 2^24 3710 against 3714; p = 127, m = 10^7 1505
+// against 1514; p = 288, m = 2^22 1397 against 1400), and at 1 to 2 GB all are
+// level.
+constexpr int64_t kFarBytes = int64_t(4) << 30;
+static bool far_inputs(const Plan* P)
+{
+    return (P->p <= 32 || P->p >= 512) && int64_t(P->p) * P->m * P->esize >= kFarBytes;
+}
+
 // On rows of 4-byte elements that are only 4-byte aligned the shared-memory
 // tile copies word by word, so the layouts beside it take over earlier
 // (graph replays, int32): the hierarchical tile in deep trees (p = 288,
@@ -340,6 +355,7 @@ int fused_launch_cols(Plan* P, const char* const* dx, char* const* dy, int64_t m
     a.tree_s = T.s;
     a.tree_slots = T.slots;
     a.tree_width = T.width;
+    a.far = vec && dx == P->d_x && !force_mode && far_inputs(P);
     a.overlap = dx == P->d_x && !force_mode;  // device buffers, no chunks between copies
     a.tree_tiles = T.width ? (a.nvec + T.width - 1) / T.width : 0;
 

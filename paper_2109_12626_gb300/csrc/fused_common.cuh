@@ -72,6 +72,7 @@ struct FusedArgs {
     int64_t tree_tiles;     // CTAs of tree_width vector units
     int tree_width;         // kTreeUnitsNarrow or kTreeUnitsWide
     int overlap;            // launch: set up while the kernel before drains
+    int far;                // inputs many times L2: FarUnit
 };
 
 template <class Op>
@@ -105,6 +106,14 @@ struct VecUnit {
     {
         st_l2(row + u * 16, v);
     }
+};
+
+// 16-byte units of inputs that are many times L2 (a.far): loads cached in L2
+// only, at normal priority.
+template <class Op>
+struct FarUnit : VecUnit<Op> {
+    __device__ __forceinline__ static uint4 ld(const char* row, int64_t u) { return ld_l2(row + u * 16); }
+    __device__ __forceinline__ static uint4 ld_wave(const char* row, int64_t u) { return ld(row, u); }
 };
 
 // Four 4-byte elements of rows that are only 4-byte aligned: columns c, c + G,
@@ -164,6 +173,7 @@ struct QuadUnit {
 
 // The wide unit of a launch: 16-byte units, or on unaligned rows of 4-byte
 // elements (a.quad) four of them; f is called with a value of the unit type.
+// with_stream_unit, of the streaming and split layouts, knows FarUnit too.
 template <class Op, int G, class F>
 inline int with_unit(const FusedArgs& a, F f)
 {
@@ -172,9 +182,15 @@ inline int with_unit(const FusedArgs& a, F f)
     }
     return f(VecUnit<Op>());
 }
+template <class Op, int G, class F>
+inline int with_stream_unit(const FusedArgs& a, F f)
+{
+    return a.far ? f(FarUnit<Op>()) : with_unit<Op, G>(a, f);
+}
 constexpr int kQuadStream = 32;  // G of the streaming and split layouts
 constexpr int kQuadTile = 8;     // of the shared-memory tile (as many units or more to a row)
 constexpr int kQuadAttr = 7;  // offset of the unaligned kernels in Plan::smem_attr
+constexpr int kFarAttr = 14;  // and of those for inputs many times L2
 
 template <class Op>
 struct OneUnit {

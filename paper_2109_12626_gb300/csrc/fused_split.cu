@@ -112,9 +112,9 @@ struct Split {
         const int64_t blocks = (units + kStreamThreads - 1) / kStreamThreads;
         const size_t smem = size_t(P->max_depth + 1) * kStreamThreads * sizeof(uint4);
         if (blocks > 0x7fffffff) return fail(DPDR_ERR_INVALID, "m too large");
-        return with_unit<Op, kQuadStream>(a, [&](auto unit) {
+        return with_stream_unit<Op, kQuadStream>(a, [&](auto unit) {
             using V = decltype(unit);
-            int* const attr = &P->smem_attr[2 + (a.quad ? kQuadAttr : 0)];
+            int* const attr = &P->smem_attr[2 + (a.quad ? kQuadAttr : a.far ? kFarAttr : 0)];
             if (int(smem) > *attr) {
                 int granted = *attr;
                 if (int rc = grant_smem(reinterpret_cast<const void*>(&fused_split_reduce_kernel<Op, V>),
