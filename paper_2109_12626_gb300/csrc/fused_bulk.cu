@@ -220,7 +220,8 @@ struct Bulk {
         const int64_t tail = (a.nvec - a.bulk_tiles * (kBulkTile / 16)) + a.nscalar;
         int64_t grid = std::min<int64_t>(a.bulk_tiles, resident);
         grid = std::max<int64_t>(grid, std::min<int64_t>(resident, (tail + kBulkConsumers - 1) / kBulkConsumers));
-        return launch_kernel(&fused_bulk_kernel<Op>, dim3(unsigned(std::max<int64_t>(grid, 1))), kBulkThreads, smem, s, a);
+        return launch_kernel(&fused_bulk_kernel<Op>, dim3(unsigned(std::max<int64_t>(grid, 1))),
+                             kBulkThreads, smem, s, a);
     }
 };
 

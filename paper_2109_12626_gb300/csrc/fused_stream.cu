@@ -119,9 +119,12 @@ struct Stream {
         if (blocks > 0x7fffffff) return fail(DPDR_ERR_INVALID, "m too large");
         return with_stream_unit<Op, kQuadStream>(a, [&](auto unit) {
             using V = decltype(unit);
-            void (*const kern)(FusedArgs) = pairs ? &fused_stream_pair_kernel<Op, V> : &fused_stream_kernel<Op, V>;
+            void (*const kern)(FusedArgs) =
+                pairs ? &fused_stream_pair_kernel<Op, V> : &fused_stream_kernel<Op, V>;
             int* const granted = &P->smem_attr[(pairs ? 6 : 0) + (a.quad ? kQuadAttr : a.far ? kFarAttr : 0)];
-            if (int rc = grant_smem(reinterpret_cast<const void*>(kern), smem, granted, "fused stream attribute")) return rc;
+            if (int rc = grant_smem(reinterpret_cast<const void*>(kern), smem, granted,
+                                    "fused stream attribute"))
+                return rc;
             return launch_kernel(kern, dim3(unsigned(blocks)), kStreamThreads, smem, s, a);
         });
     }

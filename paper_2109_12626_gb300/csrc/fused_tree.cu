@@ -150,7 +150,8 @@ struct Tree {
             const void* kern = reinterpret_cast<const void*>(&fused_tree_kernel<Op, V, W>);
             int* const granted = &P->smem_attr[(wide ? 5 : 4) + (a.quad ? kQuadAttr : 0)];
             if (int rc = grant_smem(kern, smem, granted, "fused tree attribute")) return rc;
-            return launch_kernel(&fused_tree_kernel<Op, V, W>, dim3(unsigned(blocks)), kTreeThreads, smem, s, a);
+            return launch_kernel(&fused_tree_kernel<Op, V, W>, dim3(unsigned(blocks)), kTreeThreads, smem,
+                                 s, a);
         };
         constexpr int N = kTreeUnitsNarrow, W = kTreeUnitsWide;
         return wide ? with_unit<Op, W>(a, [&](auto u) { return launch(u, std::integral_constant<int, W>()); })

@@ -523,7 +523,8 @@ extern "C" int dpdr_plan_info(dpdr_plan_t h, int64_t* info, int n)
     const int64_t v[] = {P->p, P->m, P->b, P->max_depth, fused_auto_mode(P),
                          P->sched_ctas, P->sched_ranks_per_cta,
                          int64_t(P->dmem_bytes + P->d_split_bytes + P->d_sched_bytes +
-                                 P->d_ll_bytes + P->words.bytes + P->walk.bytes + P->tree[0].bytes + P->tree[1].bytes),
+                                 P->d_ll_bytes + P->words.bytes + P->walk.bytes +
+                                 P->tree[0].bytes + P->tree[1].bytes),
                          P->last_vector_path, P->split_s, P->split_nseg, P->split_group,
                          P->sched_slices_used, P->topo, P->last_host_path,
                          schedule_transport(P), P->tree[fused_tree_index(P)].width,
