@@ -198,6 +198,16 @@ bool cell_vector(const Plan* P)
 
 int cell_tail(const Plan* P, bool vec) { return vec && P->m % (16 / int64_t(P->esize)) ? 1 : 0; }
 
+// Slots of flagged words per cell and slice, of its partial blocks and of its
+// final blocks: a power of two above the deepest rank's depth + 1
+// (schedule_words.cu, reuse of slots).
+int word_slots(const Plan* P)
+{
+    int n = 2;
+    while (n < P->max_depth + 2) n *= 2;
+    return n;
+}
+
 // The cells' device memory: control words (epoch 1 first), descriptors at 256,
 // scratch (zeroed) at off_scratch.
 int cell_scratch(Plan* P, CellPlan* C, const void* desc, size_t desc_bytes)

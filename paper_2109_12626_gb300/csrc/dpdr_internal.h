@@ -65,6 +65,7 @@ constexpr int kWalkRanks = 20, kWalkLevels = 5;
 constexpr int kCellRanks = kWalkRanks;
 constexpr int kCellLevels = kWalkLevels;
 constexpr int kCellExt = kCellRanks / 2;
+constexpr int kDualSlots = 2;  // slots of flagged words between the dual roots
 struct CellDesc {
     int n, root, depth;        // ranks, root rank and its depth
     int par_cell, par_rank;    // the root's parent, -1 at a tree's root
@@ -252,6 +253,7 @@ void make_cells(const Plan* P, int max_ranks, int max_levels, CellPlan* C, std::
 CellSlices cell_slices(const Plan* P, const CellPlan& C, bool vec);
 bool cell_vector(const Plan* P);
 int cell_tail(const Plan* P, bool vec);
+int word_slots(const Plan* P);
 int cell_scratch(Plan* P, CellPlan* C, const void* desc, size_t desc_bytes);
 int cell_launch(const void* kernel, void* args, int64_t warps, int per_cta, size_t smem, cudaStream_t s);
 int schedule_words_prepare(Plan* P);

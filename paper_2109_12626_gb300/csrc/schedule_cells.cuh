@@ -156,8 +156,9 @@ struct Spot {
 // last block in the last step of some warps (an empty extent).
 struct Pos {
     int j, g;
-    __device__ __forceinline__ Pos(const Columns& c, int slice) : j(slice / c.per_block), g(slice % c.per_block) {}
-    __device__ __forceinline__ void advance(const Columns& c)
+    __host__ __device__ __forceinline__ Pos(const Columns& c, int slice)
+        : j(slice / c.per_block), g(slice % c.per_block) {}
+    __host__ __device__ __forceinline__ void advance(const Columns& c)
     {
         for (g += c.nslices; g >= c.per_block; g -= c.per_block) j++;
     }
@@ -170,7 +171,7 @@ struct Extent {
 };
 
 template <class Op, bool kVec>
-__device__ __forceinline__ Extent extent(const Columns& c, const Pos& at, bool tail)
+__host__ __device__ __forceinline__ Extent extent(const Columns& c, const Pos& at, bool tail)
 {
     constexpr int E = Unit<Op, kVec>::kElems;
     int64_t u = sched::block_start(c.q, c.rem, at.j), e = sched::block_start(c.q, c.rem, at.j + 1);

@@ -49,7 +49,7 @@ __device__ __forceinline__ uint64_t now_ns()
 
 // First element of block j of Algorithm 1's partition of m elements into b
 // blocks (q = floor(m/b), rem = m mod b: the first rem blocks are one longer).
-__device__ __forceinline__ int64_t block_start(int64_t q, int64_t rem, int j)
+__host__ __device__ __forceinline__ int64_t block_start(int64_t q, int64_t rem, int j)
 {
     return int64_t(j) * q + lmin(j, rem);
 }

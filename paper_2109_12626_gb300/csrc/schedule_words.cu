@@ -24,9 +24,13 @@
 //   dual  2 slots: the dual's partial j + 1 shows that it has read partial j.
 //   up    depth + 1 slots: final block k shows that the parent has read
 //         partial k, and final block j - 1 - d arrived in round j - 1.
-//   down  a parent at depth d that sends final f (round f + d) has partial
-//         f + d of its child l + 1 levels below, l <= 3, which took final
-//         f - l - 2 in the round before: 5 slots, 8 used.
+//   down  depth + 1 slots of the receiving cell: final block f leaves the
+//         root only with the cell's partial block f in it, which the cell,
+//         at depth d, sent in round f, having taken final block f - 1 - d in
+//         the round before.  While partial blocks come, a parent l levels
+//         above knows of the last l + 1 rounds only and 5 slots would do; in
+//         the rounds after the last partial block nothing tells it more than
+//         that, however many final blocks it sends.
 // A cell waits in round j for its children's partial blocks j, which they
 // send before they wait for anything later than round j - 1, for the dual
 // root's partial j, sent before the wait, and for final block j - d, which its
@@ -49,7 +53,6 @@ constexpr int kLevels = kWordsLevels;
 constexpr int kExt = kRanks / 2;
 constexpr int kWarps = 4;     // per CTA
 constexpr int kNodes = 2;     // nodes that take their children's values at once
-constexpr int kDownSlots = 8;
 constexpr int kSlot = 32 * 4;  // words of a slot: 32 units of 16 bytes
 
 struct WordsArgs {
@@ -58,13 +61,13 @@ struct WordsArgs {
     const CellDesc* cells;
     uint32_t* ctl;
     uint32_t* err;
-    u64* dual;           // [2 sides][slices][2] slots: the roots' partial blocks
-    u64* down;           // [cells with children][slices][kDownSlots]: final blocks
-    u64* up;             // [cells][slices][up_slots]: partial blocks
+    u64* dual;           // [2 sides][slices][kDualSlots] slots: the roots' partial blocks
+    u64* down;           // [cells with children][slices][slots]: final blocks
+    u64* up;             // [cells][slices][slots]: partial blocks
     int64_t words;       // 32-bit words of all slots, from dual on
     Columns col;
     int64_t wait_ns;
-    int up_slots;        // a power of two above the deepest cell's depth + 1
+    int slots;           // word_slots
     int ncells, root0, root1;  // cells of the roots (root0 -1: one tree)
     int used;            // flag values the call uses
     int skip_rank;
@@ -189,7 +192,7 @@ struct Runner {
 #pragma unroll 1
         for (int q0 = 0; q0 < next; q0 += kNodes) {
             T e[2 * kNodes];
-            if (!recv<2 * kNodes>(s->up_in + 2 * q0, int64_t(t & (a.up_slots - 1)) * kSlot,
+            if (!recv<2 * kNodes>(s->up_in + 2 * q0, int64_t(t & (a.slots - 1)) * kSlot,
                                   2 * min(kNodes, next - q0), flag, p, e, j, -1))
                 return false;
             if (!landed) cp_async_wait_all();
@@ -236,10 +239,10 @@ struct Runner {
                 const uint32_t flag = s->base + uint32_t(t) + 1u;
                 if (!fold_step(t, c.j, now, v)) return;
                 if (!root) {
-                    send(s->up_out + (t & (a.up_slots - 1)) * kSlot, flag, now, v);
+                    send(s->up_out + (t & (a.slots - 1)) * kSlot, flag, now, v);
                 } else if (s->dual) {
-                    send(s->dual_out + (t & 1) * kSlot, flag, now, v);
-                    if (!recv<1>(&s->dual_in, (t & 1) * kSlot, 1, flag, now, in, c.j, 2)) return;
+                    send(s->dual_out + (t & (kDualSlots - 1)) * kSlot, flag, now, v);
+                    if (!recv<1>(&s->dual_in, (t & (kDualSlots - 1)) * kSlot, 1, flag, now, in, c.j, 2)) return;
                     v = s->cell == a.root0 ? U::op(v, in[0]) : U::op(in[0], v);
                 }
                 c.advance(a.col);
@@ -254,12 +257,12 @@ struct Runner {
                 const uint32_t flag = s->base + uint32_t(f) + 1u;
                 if (!root) {
                     now = spot<Op, kVec>(a.col, d, lane, tail);
-                    if (!recv<1>(&s->down_in, (f & (kDownSlots - 1)) * kSlot, 1, flag, now, in, d.j + D, 3))
+                    if (!recv<1>(&s->down_in, (f & (a.slots - 1)) * kSlot, 1, flag, now, in, d.j + D, 3))
                         return;
                     v = in[0];
                     d.advance(a.col);
                 }
-                if (s->next) send(s->down_out + (f & (kDownSlots - 1)) * kSlot, flag, now, v);
+                if (s->next) send(s->down_out + (f & (a.slots - 1)) * kSlot, flag, now, v);
             } else {
                 now.on = false;
             }
@@ -295,7 +298,7 @@ __global__ void __launch_bounds__(kWarps * 32, 4) words_kernel(const __grid_cons
             reinterpret_cast<uint8_t*>(&s->tape)[lane] = uint8_t(__ldg(c->tape + lane));
         }
         if (lane < 2 * kExt)
-            s->up_in[lane] = a.up + (int64_t(__ldg(c->ext_cell + lane)) * lines + g) * a.up_slots * kSlot;
+            s->up_in[lane] = a.up + (int64_t(__ldg(c->ext_cell + lane)) * lines + g) * a.slots * kSlot;
         if (lane < kExt) s->ext_k[lane] = __ldg(c->ext_k + lane);
         if (lane <= kLevels) s->lev_off[lane] = __ldg(c->lev_off + lane);
         if (lane == 31) {
@@ -309,11 +312,11 @@ __global__ void __launch_bounds__(kWarps * 32, 4) words_kernel(const __grid_cons
             s->cell = cell;
             s->g = g;
             s->dual = a.root0 >= 0 && s->par_cell < 0;
-            s->up_out = a.up + (int64_t(cell) * lines + g) * a.up_slots * kSlot;
-            s->down_in = a.down + (int64_t(__ldg(&c->par_down)) * lines + g) * kDownSlots * kSlot;
-            s->down_out = a.down + (int64_t(__ldg(&c->down)) * lines + g) * kDownSlots * kSlot;
-            s->dual_out = a.dual + (int64_t(side) * lines + g) * 2 * kSlot;
-            s->dual_in = a.dual + (int64_t(1 - side) * lines + g) * 2 * kSlot;
+            s->up_out = a.up + (int64_t(cell) * lines + g) * a.slots * kSlot;
+            s->down_in = a.down + (int64_t(__ldg(&c->par_down)) * lines + g) * a.slots * kSlot;
+            s->down_out = a.down + (int64_t(__ldg(&c->down)) * lines + g) * a.slots * kSlot;
+            s->dual_out = a.dual + (int64_t(side) * lines + g) * kDualSlots * kSlot;
+            s->dual_in = a.dual + (int64_t(1 - side) * lines + g) * kDualSlots * kSlot;
             s->mute = a.skip_rank >= 0 && s->root == a.skip_rank;
             s->stuck = -1;
             s->stuck_step = 0;
@@ -358,18 +361,10 @@ const void* words_kernel_for(int dtype, bool vec)
     }
 }
 
-// Slots for partial blocks per cell and slice.
-int up_slots(const Plan* P)
-{
-    int n = 2;
-    while (n < P->max_depth + 2) n *= 2;
-    return n;
-}
-
 size_t slot_words(const Plan* P, int lines)
 {
     return size_t(lines) * kSlot *
-           (4 + size_t(P->words.down) * kDownSlots + size_t(P->words.n) * up_slots(P));
+           (2 * kDualSlots + size_t(P->words.down + P->words.n) * word_slots(P));
 }
 
 }  // namespace
@@ -410,11 +405,11 @@ int schedule_words_launch(Plan* P, cudaStream_t s)
     a.col = Columns{P->m, P->m / P->b, P->m % P->b, P->b, S.n, S.per_block, S.steps, cell_tail(P, vec)};
     const int lines = S.n + a.col.tail;
     a.dual = reinterpret_cast<u64*>(C.d + C.off_scratch);
-    a.down = a.dual + size_t(lines) * 4 * kSlot;
-    a.up = a.down + size_t(C.down) * lines * kDownSlots * kSlot;
+    a.slots = word_slots(P);
+    a.down = a.dual + size_t(lines) * 2 * kDualSlots * kSlot;
+    a.up = a.down + size_t(C.down) * lines * a.slots * kSlot;
     a.words = int64_t(C.scratch / 4);
     a.wait_ns = P->wait_ns;
-    a.up_slots = up_slots(P);
     a.ncells = C.n;
     a.root0 = C.root0;
     a.root1 = C.root1;

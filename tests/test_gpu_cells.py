@@ -52,6 +52,8 @@ CASES = [("int32", 1, 33, (1, 4)), ("float32", 2, 1, (1,)), ("float32", 2, 4100,
          ("int32", 36, 1003, (1, 3, 400)), ("mat2x2u32", 100, 77, (1, 7)),
          ("float32", 255, 2050, (1, 16)), ("int32", 288, 250, (1, 2)),
          ("float32", 1152, 4099, (1, 6)), ("int32", 1152, 1, (1,))]
+# the same, more steps than final blocks can wait unread below a deep tree's root
+CASES += [("int32", 1025, 2048, (32,)), ("int32", 1152, 2560, (20, 40)), ("float32", 2049, 2051, (32,))]
 # counters between cells
 CASES += [("int32", 2, 1600001, (1, 5)), ("float32", 7, 500003, (1, 8, 600)),
           ("mat2x2u32", 36, 30001, (1, 7)), ("int32", 100, 40009, (1, 16, 5000)),
