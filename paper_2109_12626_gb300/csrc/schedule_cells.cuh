@@ -187,11 +187,17 @@ __host__ __device__ __forceinline__ Extent extent(const Columns& c, const Pos& a
     }
     return Extent{u, u < e && (tail || at.j < c.b) ? int(lmin(e - u, 32)) : 0};
 }
+// The first slice of a warp from `at` on that holds units, which `at` moves on
+// to: blocks differ by a unit, so a slice past the end of one block may have
+// units in the next.  False when there is none.
 template <class Op, bool kVec>
-__device__ __forceinline__ Spot spot(const Columns& c, const Pos& at, int lane, bool tail)
+__host__ __device__ __forceinline__ bool next_slice(const Columns& c, Pos& at, bool tail, Extent& x)
 {
-    const Extent x = extent<Op, kVec>(c, at, tail);
-    return Spot{(x.u + lane) * Unit<Op, kVec>::kBytes, lane < x.n};
+    for (; at.j < c.b; at.advance(c)) {
+        x = extent<Op, kVec>(c, at, tail);
+        if (x.n) return true;
+    }
+    return false;
 }
 
 // Records an expired wait (the first one of the call wins) and aborts the

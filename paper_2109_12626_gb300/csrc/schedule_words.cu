@@ -20,7 +20,9 @@
 // word travels with the step's flag in one 64-bit store and the receiver
 // polls the words themselves.  Flags never repeat (finish_call), so nothing
 // is cleared between calls and a captured graph replays.  A sender never
-// waits for a slot:
+// waits for a slot.  A warp's rounds are the slices that hold units, those
+// without are passed over, alike in every cell: so in every round each cell
+// hears from the others, which is what shows that a slot has been read.
 //   dual  2 slots: the dual's partial j + 1 shows that it has read partial j.
 //   up    depth + 1 slots: final block k shows that the parent has read
 //         partial k, and final block j - 1 - d arrived in round j - 1.
@@ -218,21 +220,31 @@ struct Runner {
             if (p.on) U::st(s->y[t] + p.off, v);
     }
 
+    // The lane's unit of the warp's next slice, from `at` on; false past the last.
+    __device__ __forceinline__ bool ahead(Pos& at, Spot& p) const
+    {
+        Extent x{0, 0};
+        const bool there = next_slice<Op, kVec>(a.col, at, tail, x);
+        p = Spot{(x.u + lane) * U::kBytes, lane < x.n};
+        return there;
+    }
+
     // A final block that reaches the cell's root in step t reaches the ranks
     // l levels below it in step t + l: the last ones wait in registers.
     __device__ __forceinline__ void run() const
     {
         static_assert(kLevels == 4, "the history of final blocks is three deep");
-        const int steps = tail ? 1 : a.col.steps, D = s->depth, nlev = s->nlev;
+        const int D = s->depth, nlev = s->nlev;
         const bool root = s->par_cell < 0;
+        int steps = tail ? 1 : a.col.steps;  // or fewer, once the last slice is seen
         Pos c(a.col, tail ? 0 : s->g), d(a.col, tail ? 0 : s->g);
-        Spot next = spot<Op, kVec>(a.col, c, lane, tail);
+        Spot next;
+        if (!ahead(c, next)) return;
         fetch(next);
         T v1{}, v2{}, v3{};
         Spot p1{0, false}, p2{0, false}, p3{0, false};
-        const int last = steps - 1 + D + nlev - 1;
 #pragma unroll 1
-        for (int t = 0; t <= last; t++) {
+        for (int t = 0; t < steps + D + nlev - 1; t++) {
             T v{}, in[1];
             Spot now = next;
             if (t < steps) {
@@ -247,8 +259,8 @@ struct Runner {
                 }
                 c.advance(a.col);
                 if (t + 1 < steps) {  // the next block's inputs
-                    next = spot<Op, kVec>(a.col, c, lane, tail);
-                    fetch(next);
+                    if (ahead(c, next)) fetch(next);
+                    else steps = t + 1;
                 }
             }
             const int f = t - D;  // the step whose block is final here now
@@ -256,7 +268,7 @@ struct Runner {
             if (f < steps) {
                 const uint32_t flag = s->base + uint32_t(f) + 1u;
                 if (!root) {
-                    now = spot<Op, kVec>(a.col, d, lane, tail);
+                    ahead(d, now);
                     if (!recv<1>(&s->down_in, (f & (a.slots - 1)) * kSlot, 1, flag, now, in, d.j + D, 3))
                         return;
                     v = in[0];

@@ -29,15 +29,20 @@ struct Op {
     int seq;             // the step whose block travels
 };
 
-// Steps of line g that hold units, by the step's number.
+// The rounds of line g, and whether its slice of the round holds units: the
+// kernel's have one each; with `empty` those without are rounds, too.
 template <class T, bool kVec>
-std::vector<char> live_steps(const cells::Columns& c, int g)
+std::vector<char> line_rounds(const cells::Columns& c, int g, bool empty)
 {
+    if (g == c.nslices) return {1};  // the tail
     std::vector<char> live;
-    if (c.tail && g == c.nslices) return {1};
-    cells::Pos at(c, g);
-    for (int t = 0; t < c.steps; t++, at.advance(c))
-        live.push_back(cells::extent<T, kVec>(c, at, false).n > 0);
+    cells::Extent x;
+    if (empty)
+        for (cells::Pos at(c, g); at.j < c.b; at.advance(c))
+            live.push_back(cells::extent<T, kVec>(c, at, false).n > 0);
+    else
+        for (cells::Pos at(c, g); cells::next_slice<T, kVec>(c, at, false, x); at.advance(c))
+            live.push_back(1);
     return live;
 }
 
@@ -48,7 +53,7 @@ std::vector<Op> program(const std::vector<CellDesc>& cells, const CellPlan& C, i
     const int steps = int(live.size()), D = c.depth;
     const bool root = c.par_cell < 0, dual = root && C.root0 >= 0;
     std::vector<Op> ops;
-    for (int t = 0; t <= steps - 1 + D + c.nlev - 1; t++) {
+    for (int t = 0; steps && t < steps + D + c.nlev - 1; t++) {
         if (t < steps && live[t]) {
             for (int h = 0; h < 2 * c.next; h++) ops.push_back({false, kUp, c.ext_cell[h], t});
             if (!root) ops.push_back({true, kUp, me, t});
@@ -126,18 +131,14 @@ int replay(const std::vector<CellDesc>& cells, const CellPlan& C, const std::vec
     return 0;
 }
 
-template <class T>
-std::vector<char> live_of(const cells::Columns& c, int g, bool vec)
-{
-    return vec ? live_steps<T, true>(c, g) : live_steps<T, false>(c, g);
-}
-
 }  // namespace
 
-// Every kind of line of a call on `warps` resident warps; out: {steps of the
-// longest line, cells, depth of the deepest cell} and, after a failure, where.
+// Every line of a call on `warps` resident warps: 0, what replay returns, 3
+// more steps than the call counts on, 4 the cells do not fit; out: {steps of
+// the longest line, cells, depth of the deepest cell} and where it failed.
+// down_slots (0: the kernel's) and empty change the kernel's rules.
 extern "C" int words_protocol(int p, int64_t m, int esize, int single, int b, int aligned, int warps,
-                              int* out)
+                              int down_slots, int empty, int* out)
 {
     Plan P;
     P.p = p;
@@ -158,10 +159,11 @@ extern "C" int words_protocol(int p, int64_t m, int esize, int single, int b, in
     std::vector<CellDesc> cells;
     make_cells(&P, kWordsRanks, kWordsLevels, &C, &cells);
     C.warps = warps;
+    if (2 * C.n > warps) return 4;
     const bool vec = cell_vector(&P);
     const CellSlices S = cell_slices(&P, C, vec);
     const cells::Columns c{m, m / b, m % b, b, S.n, S.per_block, S.steps, cell_tail(&P, vec)};
-    const int slots[3] = {word_slots(&P), word_slots(&P), kDualSlots};
+    const int slots[3] = {word_slots(&P), down_slots ? down_slots : word_slots(&P), kDualSlots};
     out[0] = 0;
     out[1] = C.n;
     out[2] = 0;
@@ -169,8 +171,10 @@ extern "C" int words_protocol(int p, int64_t m, int esize, int single, int b, in
     std::map<std::vector<char>, bool> seen;
     for (int g = 0; g < S.n + c.tail; g++) {
         const std::vector<char> live =
-            esize == 4 ? live_of<SumI32>(c, g, vec) : live_of<MatU32>(c, g, vec);
-        out[0] = std::max(out[0], int(std::count(live.begin(), live.end(), 1)));
+            esize == 4 ? (vec ? line_rounds<SumI32, true>(c, g, empty) : line_rounds<SumI32, false>(c, g, empty))
+                       : (vec ? line_rounds<MatU32, true>(c, g, empty) : line_rounds<MatU32, false>(c, g, empty));
+        if (int(live.size()) > S.steps) return 3;  // more than the call's flags
+        out[0] = std::max(out[0], int(live.size()));
         if (seen[live]) continue;
         seen[live] = true;
         if (const int bad = replay(cells, C, live, slots, out + 3)) return bad;

@@ -54,6 +54,9 @@ CASES = [("int32", 1, 33, (1, 4)), ("float32", 2, 1, (1,)), ("float32", 2, 4100,
          ("float32", 1152, 4099, (1, 6)), ("int32", 1152, 1, (1,))]
 # the same, more steps than final blocks can wait unread below a deep tree's root
 CASES += [("int32", 1025, 2048, (32,)), ("int32", 1152, 2560, (20, 40)), ("float32", 2049, 2051, (32,))]
+# the same, blocks whose last slice holds units in some and none in others
+CASES += [("int32", 2, 2064, (16,)), ("float32", 36, 2064, (16,)), ("int32", 288, 2064, (16,)),
+          ("int32", 36, 653, (20,)), ("mat2x2u32", 7, 653, (20,))]
 # counters between cells
 CASES += [("int32", 2, 1600001, (1, 5)), ("float32", 7, 500003, (1, 8, 600)),
           ("mat2x2u32", 36, 30001, (1, 7)), ("int32", 100, 40009, (1, 16, 5000)),
