@@ -3,8 +3,7 @@
 // slices, scratch and launches (schedule_cells.cuh, schedule_words.cu,
 // schedule_walk.cu).
 #include <algorithm>
-#include <cstring>
-#include <map>
+#include <utility>
 
 #include "dpdr_internal.h"
 
@@ -21,151 +20,155 @@ struct Cut {
 };
 constexpr int kNoCut = 1 << 28;
 
-struct HostCell {
-    std::vector<int> ranks;  // post-order, the cell's root last
-    int root, depth, par_cell, par_rank, nlev;
+// A cut of the plan's trees.  Cells are numbered by their root ranks, so
+// that child cells come before their parents' cells.
+struct Cells {
+    std::vector<int> cell, pos;     // of each rank: its cell, its place in the cell's post-order
+    std::vector<char> top;          // whether it is the cell's root
+    std::vector<int> first, ranks;  // cell k: ranks[first[k]] .. ranks[first[k + 1] - 1]
 };
 
-// The cells of the plan's trees.  A node's children are both in its cell or
+// The cells of the plan's trees, and how many (returned); when they are more
+// than max_cells, that alone.  A node's children are both in its cell or
 // both roots of other cells, and a cell holds at most max_ranks ranks on
 // max_levels levels.  Of all such cuts: the fewest cells between a leaf and
 // the root (each costs an exchange through L2 each way), then the fewest
 // cells.  Subtrees of a complete tree that have the same size have the same
 // shape, so the best cut is found once per size; pieces are numbered
 // (ranks - 1) * max_levels + (levels - 1).
-void cut_cells(const Plan* P, int max_ranks, int max_levels, std::vector<HostCell>* cells,
-               std::vector<int>* cell_of, std::vector<char>* top_of)
+int cut_cells(const Plan* P, int max_ranks, int max_levels, int max_cells, Cells* out)
 {
     const int p = P->p, pieces = max_ranks * max_levels;
-    std::vector<int> size(p), piece(p, 0);
-    std::vector<int>& cell = *cell_of;
-    std::vector<char>& top = *top_of;
-    cell.assign(p, -1);
-    top.assign(p, 0);
-    std::map<int, std::vector<Cut>> cuts;
-    auto best = [](const std::vector<Cut>& c) { return int(std::min_element(c.begin(), c.end()) - c.begin()); };
+    std::vector<int> size(p), shape_of(p + 1, -1), best;  // a size's shape, a shape's best piece
+    std::vector<std::vector<Cut>> cuts;                   // by shape
     for (int i = 0; i < p; i++) {  // post-order: children first
         const int c0 = P->child0[i], c1 = P->child1[i];
         size[i] = 1 + (c0 >= 0 ? size[c0] : 0) + (c1 >= 0 ? size[c1] : 0);
-        std::vector<Cut>& c = cuts[size[i]];
-        if (!c.empty()) continue;
-        c.assign(pieces, Cut{kNoCut, 0, false, 0, 0});
+        if (shape_of[size[i]] >= 0) continue;
+        std::vector<Cut> c(pieces, Cut{kNoCut, 0, false, 0, 0});
         if (c0 < 0) {
             c[0] = Cut{0, 0, false, 0, 0};
-            continue;
-        }
-        const std::vector<Cut>& a = cuts[size[c0]];
-        const std::vector<Cut>& d = c1 >= 0 ? cuts[size[c1]] : a;
-        if (c1 >= 0) {
-            const Cut x = a[best(a)], y = d[best(d)];
-            c[0] = Cut{1 + std::max(x.tiers, y.tiers), 2 + x.cells + y.cells, false, 0, 0};
-        }
-        for (int s0 = 0; s0 < pieces; s0++) {
-            if (a[s0].tiers >= kNoCut) continue;
-            for (int s1 = 0; s1 < (c1 >= 0 ? pieces : 1); s1++) {
-                const Cut x = a[s0], y = c1 >= 0 ? d[s1] : Cut{0, 0, false, 0, 0};
-                if (y.tiers >= kNoCut) continue;
-                const int n = 1 + s0 / max_levels + 1 + (c1 >= 0 ? s1 / max_levels + 1 : 0);
-                const int l = 1 + std::max(s0 % max_levels + 1, c1 >= 0 ? s1 % max_levels + 1 : 0);
-                if (n > max_ranks || l > max_levels) continue;
-                Cut& b = c[(n - 1) * max_levels + l - 1];
-                const Cut j{std::max(x.tiers, y.tiers), x.cells + y.cells, true, s0, s1};
-                if (j < b) b = j;
+        } else {
+            const int sa = shape_of[size[c0]], sd = c1 >= 0 ? shape_of[size[c1]] : sa;
+            const std::vector<Cut>&a = cuts[sa], &d = cuts[sd];
+            if (c1 >= 0) {
+                const Cut x = a[best[sa]], y = d[best[sd]];
+                c[0] = Cut{1 + std::max(x.tiers, y.tiers), 2 + x.cells + y.cells, false, 0, 0};
+            }
+            for (int s0 = 0; s0 < pieces; s0++) {
+                if (a[s0].tiers >= kNoCut) continue;
+                for (int s1 = 0; s1 < (c1 >= 0 ? pieces : 1); s1++) {
+                    const Cut x = a[s0], y = c1 >= 0 ? d[s1] : Cut{0, 0, false, 0, 0};
+                    if (y.tiers >= kNoCut) continue;
+                    const int n = 1 + s0 / max_levels + 1 + (c1 >= 0 ? s1 / max_levels + 1 : 0);
+                    const int l = 1 + std::max(s0 % max_levels + 1, c1 >= 0 ? s1 % max_levels + 1 : 0);
+                    if (n > max_ranks || l > max_levels) continue;
+                    Cut& b = c[(n - 1) * max_levels + l - 1];
+                    const Cut j{std::max(x.tiers, y.tiers), x.cells + y.cells, true, s0, s1};
+                    if (j < b) b = j;
+                }
             }
         }
+        shape_of[size[i]] = int(cuts.size());
+        best.push_back(int(std::min_element(c.begin(), c.end()) - c.begin()));
+        cuts.push_back(std::move(c));
     }
+    auto cells_below = [&](int i) { return cuts[shape_of[size[i]]][best[shape_of[size[i]]]].cells; };
+    const int n = 1 + cells_below(P->r1) + (P->r0 >= 0 ? 1 + cells_below(P->r0) : 0);
+    if (n > max_cells) return n;
+
+    std::vector<int> piece(p, 0);
+    out->top.assign(p, 0);
     for (int i = p - 1; i >= 0; i--) {  // parents first: the pieces chosen
-        if (P->parent[i] < 0) top[i] = 1;
-        const std::vector<Cut>& c = cuts[size[i]];
-        if (top[i]) piece[i] = best(c);
+        const int shape = shape_of[size[i]];
+        if (P->parent[i] < 0) out->top[i] = 1;
+        if (out->top[i]) piece[i] = best[shape];
         const int c0 = P->child0[i], c1 = P->child1[i];
         if (c0 < 0) continue;
-        const Cut& k = c[piece[i]];
-        top[c0] = !k.join;
+        const Cut& k = cuts[shape][piece[i]];
+        out->top[c0] = !k.join;
         piece[c0] = k.s0;
         if (c1 >= 0) {
-            top[c1] = !k.join;
+            out->top[c1] = !k.join;
             piece[c1] = k.s1;
         }
     }
-    cells->clear();
-    for (int i = 0; i < p; i++)
-        if (top[i]) {
-            cell[i] = int(cells->size());
-            cells->push_back(HostCell());
-        }
-    for (int i = p - 1; i >= 0; i--)
-        if (cell[i] < 0) cell[i] = cell[P->parent[i]];
-    for (int i = 0; i < p; i++) (*cells)[cell[i]].ranks.push_back(i);
-    for (HostCell& c : *cells) {
-        c.root = c.ranks.back();
-        c.depth = P->depth[c.root];
-        c.par_rank = P->parent[c.root];
-        c.par_cell = c.par_rank < 0 ? -1 : cell[c.par_rank];
-        c.nlev = 0;
-        for (int i : c.ranks) c.nlev = std::max(c.nlev, P->depth[i] - c.depth + 1);
+    out->cell.resize(p);
+    out->first.assign(n + 1, 0);
+    for (int i = p - 1, k = n; i >= 0; i--) {
+        out->cell[i] = out->top[i] ? --k : out->cell[P->parent[i]];
+        out->first[out->cell[i] + 1]++;
     }
+    for (int k = 0; k < n; k++) out->first[k + 1] += out->first[k];
+    std::vector<int> held(n, 0);
+    out->pos.resize(p);
+    out->ranks.resize(p);
+    for (int i = 0; i < p; i++) {  // the cell's root is its last rank
+        const int k = out->cell[i];
+        out->pos[i] = held[k]++;
+        out->ranks[out->first[k] + out->pos[i]] = i;
+    }
+    return n;
 }
 
 bool is_second(const Plan* P, int i) { return P->parent[i] >= 0 && P->child1[P->parent[i]] == i; }
 
 }  // namespace
 
-void make_cells(const Plan* P, int max_ranks, int max_levels, CellPlan* C, std::vector<CellDesc>* out)
+// The cells' descriptors; false when there are more than max_cells of them.
+bool make_cells(const Plan* P, int max_ranks, int max_levels, int max_cells, CellPlan* C,
+                std::vector<CellDesc>* out)
 {
-    std::vector<HostCell> cells;
-    std::vector<int> cell;
-    std::vector<char> top;
-    cut_cells(P, max_ranks, max_levels, &cells, &cell, &top);
-    out->assign(cells.size(), CellDesc());
-    C->n = int(cells.size());
-    C->root0 = P->r0 >= 0 ? cell[P->r0] : -1;
-    C->root1 = cell[P->r1];
+    Cells cells;
+    C->n = cut_cells(P, max_ranks, max_levels, max_cells, &cells);
+    out->clear();
+    if (C->n > max_cells) return false;
+    out->resize(C->n);  // zeros
+    C->root0 = P->r0 >= 0 ? cells.cell[P->r0] : -1;
+    C->root1 = cells.cell[P->r1];
     C->down = C->ranks = 0;
-    for (size_t k = 0; k < cells.size(); k++) {
-        const HostCell& h = cells[k];
+    for (int k = 0; k < C->n; k++) {
+        const int* const ranks = cells.ranks.data() + cells.first[k];
         CellDesc& c = (*out)[k];
-        std::memset(&c, 0, sizeof c);
-        c.n = int(h.ranks.size());
+        c.n = cells.first[k + 1] - cells.first[k];
         C->ranks = std::max(C->ranks, c.n);
-        c.root = h.root;
-        c.depth = h.depth;
-        c.par_cell = h.par_cell;
-        c.par_rank = h.par_rank;
-        c.nlev = h.nlev;
+        c.root = ranks[c.n - 1];
+        c.depth = P->depth[c.root];
+        c.par_rank = P->parent[c.root];
+        c.par_cell = c.par_rank < 0 ? -1 : cells.cell[c.par_rank];
         unsigned again = 0;  // positions whose final blocks child cells read
         for (int t = 0; t < c.n; t++) {
-            const int i = h.ranks[t], c0 = P->child0[i], c1 = P->child1[i];
-            const bool in = c0 >= 0 && !top[c0];
-            const int pos1 = in && c1 >= 0
-                ? int(std::find(h.ranks.begin(), h.ranks.end(), c1) - h.ranks.begin()) : 0;
+            const int i = ranks[t], c0 = P->child0[i], c1 = P->child1[i];
+            const bool in = c0 >= 0 && !cells.top[c0];
+            const int pos1 = in && c1 >= 0 ? cells.pos[c1] : 0;
+            c.nlev = std::max(c.nlev, P->depth[i] - c.depth + 1);
+            c.lev_off[P->depth[i] - c.depth + 1]++;
             c.rank[t] = i;
-            c.node_par[t] = i == h.root ? -1 : P->parent[i];
-            c.tape[t] = (in ? (c1 >= 0 ? 2 : 1) : 0) | (i != h.root && is_second(P, i) ? 4 : 0) |
+            c.node_par[t] = i == c.root ? -1 : P->parent[i];
+            c.tape[t] = (in ? (c1 >= 0 ? 2 : 1) : 0) | (i != c.root && is_second(P, i) ? 4 : 0) |
                         (pos1 << 3);
             if (c0 >= 0 && !in) {  // two children: a single one always joins
                 c.ext_k[c.next] = t;
-                c.ext_cell[2 * c.next] = cell[c0];
-                c.ext_cell[2 * c.next + 1] = cell[c1];
+                c.ext_cell[2 * c.next] = cells.cell[c0];
+                c.ext_cell[2 * c.next + 1] = cells.cell[c1];
                 c.ext_rank[2 * c.next] = c0;
                 c.ext_rank[2 * c.next + 1] = c1;
                 c.next++;
                 again |= 1u << t;
             }
         }
-        int t = 0;
-        for (int l = 0; l < kCellLevels; l++) {
-            c.lev_off[l] = t;
-            for (int q = 0; q < c.n; q++)
-                if (P->depth[h.ranks[q]] - h.depth == l) {
-                    if ((again >> q) & 1u) c.reread |= 1 << t;
-                    c.lev_k[t++] = q;
-                }
+        for (int l = 0; l < kCellLevels; l++) c.lev_off[l + 1] += c.lev_off[l];
+        int at[kCellLevels];
+        std::copy(c.lev_off, c.lev_off + kCellLevels, at);
+        for (int q = 0; q < c.n; q++) {
+            const int t = at[P->depth[ranks[q]] - c.depth]++;
+            c.lev_k[t] = q;
+            c.reread |= int((again >> q) & 1u) << t;
         }
-        c.lev_off[kCellLevels] = t;
         c.down = c.next ? C->down++ : 0;
     }
     for (CellDesc& c : *out) c.par_down = c.par_cell < 0 ? 0 : (*out)[c.par_cell].down;
+    return true;
 }
 
 // Slices of 32 units, those of all blocks one after another, dealt out to the
@@ -225,12 +228,10 @@ int cell_scratch(Plan* P, CellPlan* C, const void* desc, size_t desc_bytes)
         }
         C->bytes = bytes;
     }
-    std::vector<char> head(256 + desc_bytes, 0);
-    const uint32_t one = 1;
-    std::memcpy(head.data(), &one, sizeof one);
-    std::memcpy(head.data() + 256, desc, desc_bytes);
-    e = cudaMemset(C->d + C->off_scratch, 0, C->scratch);
-    if (e == cudaSuccess) e = cudaMemcpy(C->d, head.data(), head.size(), cudaMemcpyHostToDevice);
+    e = cudaMemset(C->d, 0, 256);
+    if (e == cudaSuccess) e = cudaMemset(C->d, 1, 1);  // the epoch's low byte
+    if (e == cudaSuccess) e = cudaMemset(C->d + C->off_scratch, 0, C->scratch);
+    if (e == cudaSuccess) e = cudaMemcpy(C->d + 256, desc, desc_bytes, cudaMemcpyHostToDevice);
     return e == cudaSuccess ? DPDR_OK : cuda_fail(e, "schedule cells: upload");
 }
 

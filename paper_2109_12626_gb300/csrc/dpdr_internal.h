@@ -249,7 +249,8 @@ int schedule_configure(Plan* P);                // schedule.cu
 // schedule_walk.cu)
 int schedule_cells_prepare(Plan* P);
 const CellPlan* schedule_cells(const Plan* P, int algo);  // the cells algo runs on, or null
-void make_cells(const Plan* P, int max_ranks, int max_levels, CellPlan* C, std::vector<CellDesc>* out);
+bool make_cells(const Plan* P, int max_ranks, int max_levels, int max_cells, CellPlan* C,
+                std::vector<CellDesc>* out);
 CellSlices cell_slices(const Plan* P, const CellPlan& C, bool vec);
 bool cell_vector(const Plan* P);
 int cell_tail(const Plan* P, bool vec);

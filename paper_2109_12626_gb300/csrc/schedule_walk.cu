@@ -14,6 +14,8 @@ const void* kernel(int dtype, bool vec, int algo)
     return algo ? walk_reduce_bcast_kernel(dtype, vec) : walk::kernel_for<false>(dtype, vec);
 }
 
+constexpr int kMaxWarpsPerSm = 64;
+
 }  // namespace
 
 int schedule_walk_prepare(Plan* P)
@@ -26,7 +28,10 @@ int schedule_walk_prepare(Plan* P)
     // longer: p = 1152, m = 2^16 int32 15 % slower).
     const int tree = P->r0 >= 0 ? P->p - P->p / 2 : P->p;
     std::vector<CellDesc> desc;
-    make_cells(P, tree <= walk::kRanks ? walk::kRanks : 16, walk::kLevels, &C, &desc);
+    if (P->max_depth + 1 >= walk::kPast) return DPDR_OK;
+    if (!make_cells(P, tree <= walk::kRanks ? walk::kRanks : 16, walk::kLevels, kMaxWarpsPerSm * P->num_sms / 2, &C,
+                    &desc))
+        return DPDR_OK;
     int occ = 1 << 20;
     for (int algo = 0; algo < (P->topo == DPDR_TOPO_SINGLE ? 2 : 1); algo++)
         for (bool vec : {false, true}) {
@@ -40,7 +45,7 @@ int schedule_walk_prepare(Plan* P)
             occ = std::min(occ, o);
         }
     C.warps = occ * P->num_sms * walk::kWarps;
-    if (2 * C.n > C.warps || P->max_depth + 1 >= walk::kPast) return DPDR_OK;  // a slice and the tail do not fit
+    if (2 * C.n > C.warps) return DPDR_OK;  // a slice and the tail do not fit
     const int lines = 1 + std::max(cell_slices(P, C, false).n, cell_slices(P, C, true).n);
     const size_t counters = sizeof(uint32_t) * walk::kCtr * 2 * size_t(C.n) * lines;
     C.off_scratch = 256 + (sizeof(CellDesc) * desc.size() + 255) / 256 * 256;

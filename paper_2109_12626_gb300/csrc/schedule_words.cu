@@ -385,8 +385,6 @@ int schedule_words_prepare(Plan* P)
 {
     CellPlan& C = P->words;
     C.ready = false;
-    std::vector<CellDesc> desc;
-    make_cells(P, kRanks, kLevels, &C, &desc);
     int occ[2] = {0, 0};
     for (int vec = 0; vec < 2; vec++) {
         const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
@@ -394,7 +392,8 @@ int schedule_words_prepare(Plan* P)
         if (e != cudaSuccess) return cuda_fail(e, "schedule words: occupancy");
     }
     C.warps = std::min(occ[0], occ[1]) * P->num_sms * kWarps;
-    if (2 * C.n > C.warps) return DPDR_OK;  // one slice and the tail do not fit
+    std::vector<CellDesc> desc;
+    if (!make_cells(P, kRanks, kLevels, C.warps / 2, &C, &desc)) return DPDR_OK;  // a slice and the tail do not fit
     const int lines = 1 + std::max(cell_slices(P, C, false).n, cell_slices(P, C, true).n);
     C.off_scratch = 256 + (sizeof(CellDesc) * desc.size() + 255) / 256 * 256;
     C.scratch = slot_words(P, lines) * sizeof(u64);

@@ -157,15 +157,15 @@ extern "C" int words_protocol(int p, int64_t m, int esize, int single, int b, in
     P.r1 = p - 1;
     CellPlan C;
     std::vector<CellDesc> cells;
-    make_cells(&P, kWordsRanks, kWordsLevels, &C, &cells);
     C.warps = warps;
-    if (2 * C.n > warps) return 4;
+    const bool fit = make_cells(&P, kWordsRanks, kWordsLevels, warps / 2, &C, &cells);
+    out[1] = C.n;
+    if (!fit) return 4;
     const bool vec = cell_vector(&P);
     const CellSlices S = cell_slices(&P, C, vec);
     const cells::Columns c{m, m / b, m % b, b, S.n, S.per_block, S.steps, cell_tail(&P, vec)};
     const int slots[3] = {word_slots(&P), down_slots ? down_slots : word_slots(&P), kDualSlots};
     out[0] = 0;
-    out[1] = C.n;
     out[2] = 0;
     for (const CellDesc& d : cells) out[2] = std::max(out[2], d.depth);
     std::map<std::vector<char>, bool> seen;

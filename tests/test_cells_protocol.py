@@ -66,3 +66,11 @@ def test_replay_sees_slots_written_too_soon(replay):
         replay(p, 512, 4, single, 8, True, down_slots=8)
     for p in (2, 32, 36, 288):
         replay(p, 2064, 4, False, 16, True, empty=True, bad=1)
+
+
+def test_more_cells_than_fit(replay):
+    """Two warps per cell are the least (a slice and the tail): with more
+    cells than that the cut is given up before any cell is laid out."""
+    for p, cells in ((20000, 2866), (9000, 1294)):
+        assert replay(p, 1000, 4, False, 1, True, bad=4)["cells"] == cells
+    assert replay(8000, 1000, 4, False, 1, True)["cells"] <= 1216
