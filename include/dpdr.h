@@ -121,10 +121,11 @@ int dpdr_block_count_rule(int p, int64_t m, double kappa);
 
 /* Builds the trees, the block partition and the device tables for p ranks
  * of m elements of (dtype, op) on the current CUDA device, and allocates the
- * plan's device scratch (rank-pointer tables, handshake counters, the dual
- * roots' exchange slots, an error word, and the cell tables, counters and
- * word slots of the schedule kernels on subtree cells; the word arrays of
- * the flagged-word transport without cells when that is selected).  b is the
+ * plan's device scratch (rank-pointer tables, an error word, and the cell
+ * tables, counters or word slots of the schedule kernels on subtree cells;
+ * where they do not run on cells, from the start or once an option asks for
+ * another layout, its tables, handshake counters, the dual roots' exchange
+ * slots, or the word arrays of the flagged-word transport).  b is the
  * number of pipeline blocks (Algorithm 1), clamped to [1, max(m,1)].
  * b == 0 selects a block count measured for the schedule kernel on this
  * GPU: 1 when the flagged-word transport is selected (latency-bound);

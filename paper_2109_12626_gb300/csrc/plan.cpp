@@ -291,7 +291,6 @@ static int allocate(Plan* P)
     const size_t o_lo = carve(sizeof(int) * P->level_off.size());
     const size_t o_tab = carve(sizeof(int) * 4 * size_t(p));
     const size_t o_err = carve(sizeof(uint32_t) * 4);
-    const size_t o_ring = carve(4 * P->ring_slot_bytes);
     P->dmem_bytes = off;
     cudaError_t e = cudaMalloc(&P->dmem, off);
     if (e != cudaSuccess) return cuda_fail(e, "dpdr_plan: cudaMalloc");
@@ -303,7 +302,6 @@ static int allocate(Plan* P)
     P->d_level_off = reinterpret_cast<int*>(base + o_lo);
     P->d_tables = reinterpret_cast<int*>(base + o_tab);
     P->d_err = reinterpret_cast<uint32_t*>(base + o_err);
-    P->d_ring = base + o_ring;
 
     std::vector<int> tab(size_t(4) * p);
     std::copy(P->parent.begin(), P->parent.end(), tab.begin());

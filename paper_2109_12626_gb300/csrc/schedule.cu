@@ -1131,7 +1131,8 @@ int schedule_configure(Plan* P)
         if (es != cudaSuccess) return cuda_fail(es, "schedule shared memory");
     }
     P->sched_ranks_per_cta = words || layout == 1 ? R : L.max_ranks;
-    // on cells, the tables and counters of the layout above are not needed
+    // on cells, the tables, counters and exchange slots of the layout above
+    // are not needed
     rc = schedule_cells_prepare(P);
     if (rc) return rc;
     if (schedule_cells(P, 0) && (P->topo == DPDR_TOPO_DUAL || schedule_cells(P, 1))) return DPDR_OK;
@@ -1139,7 +1140,8 @@ int schedule_configure(Plan* P)
     const size_t off_first = (words_n * sizeof(uint32_t) + 255) / 256 * 256;
     const size_t off_groups = (off_first + sizeof(int) * first.size() + 255) / 256 * 256;
     const size_t off_ranks = off_groups + sizeof(int4) * L.groups.size();
-    const size_t bytes = off_ranks + sizeof(int) * L.ranks.size() + 16;
+    const size_t off_ring = (off_ranks + sizeof(int) * L.ranks.size() + 16 + 255) / 256 * 256;
+    const size_t bytes = off_ring + 4 * P->ring_slot_bytes;
     cudaError_t e;
     if (bytes > P->d_sched_bytes) {
         if (P->d_sched) cudaFree(P->d_sched);
@@ -1153,6 +1155,7 @@ int schedule_configure(Plan* P)
     P->d_cta_first = reinterpret_cast<int*>(P->d_sched + off_first);
     P->d_groups = reinterpret_cast<int4*>(P->d_sched + off_groups);
     P->d_rank_list = reinterpret_cast<int*>(P->d_sched + off_ranks);
+    P->d_ring = P->d_sched + off_ring;
     e = cudaMemcpy(P->d_cta_first, first.data(), sizeof(int) * first.size(),
                    cudaMemcpyHostToDevice);
     if (e == cudaSuccess && !L.groups.empty())

@@ -103,6 +103,26 @@ def test_cells_choice(pkg):
         assert plan.info()["sched_cells"] == 0
 
 
+def test_cells_take_the_place_of_other_scratch(pkg, orc):
+    """A plan on cells holds nothing of the kernels that they replace: the
+    dual roots' exchange slots (four of a block each) come with the option
+    that asks for those."""
+    kind, p, m = "mat2x2u32", 36, 65536
+    x = host_inputs(kind, 104, p, m)
+    want = expect_bits(orc.tree_fold(x, orc.MAT, orc.DUAL))
+    xs, _ = to_device(x, kind, torch.device("cuda:0"))
+    with pkg.Plan(p, m, kind, 1) as plan:
+        held = []
+        for transport in (0, 1, 0, 1):
+            plan.set(pkg.OPT_SCHED_TRANSPORT, transport)
+            held.append(plan.info()["scratch_bytes"])
+            ys, _k = empty_like_ranks(xs)
+            plan.allreduce_schedule(xs, ys)
+            plan.sync()
+            _check(ys, want, "transport %d" % transport)
+        assert held[1] - held[0] >= 4 * 16 * m and held[1] == held[2] == held[3]
+
+
 def test_cells_change_of_options_and_alignment(pkg, orc):
     """One plan, calls of different kinds in a row: aligned and unaligned
     buffers (other slice counts over the same counters), other block counts,
