@@ -202,12 +202,13 @@ bool cell_vector(const Plan* P)
 int cell_tail(const Plan* P, bool vec) { return vec && P->m % (16 / int64_t(P->esize)) ? 1 : 0; }
 
 // Slots of flagged words per cell and slice, of its partial blocks and of its
-// final blocks: a power of two above the deepest rank's depth + 1
-// (schedule_words.cu, reuse of slots).
-int word_slots(const Plan* P)
+// final blocks, in a call of so many steps: a power of two above the deepest
+// rank's depth + 1 (schedule_words.cu, reuse of slots), or of at least one
+// slot per step.
+int word_slots(const Plan* P, int steps)
 {
-    int n = 2;
-    while (n < P->max_depth + 2) n *= 2;
+    int n = 1;
+    while (n < P->max_depth + 2 && n < steps) n *= 2;
     return n;
 }
 

@@ -254,7 +254,7 @@ bool make_cells(const Plan* P, int max_ranks, int max_levels, int max_cells, Cel
 CellSlices cell_slices(const Plan* P, const CellPlan& C, bool vec);
 bool cell_vector(const Plan* P);
 int cell_tail(const Plan* P, bool vec);
-int word_slots(const Plan* P);
+int word_slots(const Plan* P, int steps);
 int cell_scratch(Plan* P, CellPlan* C, const void* desc, size_t desc_bytes);
 int cell_launch(const void* kernel, void* args, int64_t warps, int per_cta, size_t smem, cudaStream_t s);
 int schedule_words_prepare(Plan* P);

@@ -373,10 +373,11 @@ const void* words_kernel_for(int dtype, bool vec)
     }
 }
 
-size_t slot_words(const Plan* P, int lines)
+// 64-bit words of the slots of a call on S.n slices and the tail.
+size_t slot_words(const Plan* P, const CellSlices& S)
 {
-    return size_t(lines) * kSlot *
-           (2 * kDualSlots + size_t(P->words.down + P->words.n) * word_slots(P));
+    return size_t(S.n + 1) * kSlot *
+           (2 * kDualSlots + size_t(P->words.down + P->words.n) * word_slots(P, S.steps));
 }
 
 }  // namespace
@@ -394,9 +395,9 @@ int schedule_words_prepare(Plan* P)
     C.warps = std::min(occ[0], occ[1]) * P->num_sms * kWarps;
     std::vector<CellDesc> desc;
     if (!make_cells(P, kRanks, kLevels, C.warps / 2, &C, &desc)) return DPDR_OK;  // a slice and the tail do not fit
-    const int lines = 1 + std::max(cell_slices(P, C, false).n, cell_slices(P, C, true).n);
     C.off_scratch = 256 + (sizeof(CellDesc) * desc.size() + 255) / 256 * 256;
-    C.scratch = slot_words(P, lines) * sizeof(u64);
+    C.scratch = std::max(slot_words(P, cell_slices(P, C, false)), slot_words(P, cell_slices(P, C, true))) *
+                sizeof(u64);
     const int rc = cell_scratch(P, &C, desc.data(), sizeof(CellDesc) * desc.size());
     C.ready = rc == DPDR_OK;
     return rc;
@@ -416,7 +417,7 @@ int schedule_words_launch(Plan* P, cudaStream_t s)
     a.col = Columns{P->m, P->m / P->b, P->m % P->b, P->b, S.n, S.per_block, S.steps, cell_tail(P, vec)};
     const int lines = S.n + a.col.tail;
     a.dual = reinterpret_cast<u64*>(C.d + C.off_scratch);
-    a.slots = word_slots(P);
+    a.slots = word_slots(P, S.steps);
     a.down = a.dual + size_t(lines) * 2 * kDualSlots * kSlot;
     a.up = a.down + size_t(C.down) * lines * a.slots * kSlot;
     a.words = int64_t(C.scratch / 4);

@@ -164,7 +164,8 @@ extern "C" int words_protocol(int p, int64_t m, int esize, int single, int b, in
     const bool vec = cell_vector(&P);
     const CellSlices S = cell_slices(&P, C, vec);
     const cells::Columns c{m, m / b, m % b, b, S.n, S.per_block, S.steps, cell_tail(&P, vec)};
-    const int slots[3] = {word_slots(&P), down_slots ? down_slots : word_slots(&P), kDualSlots};
+    const int slots[3] = {word_slots(&P, S.steps), down_slots ? down_slots : word_slots(&P, S.steps),
+                          kDualSlots};
     out[0] = 0;
     out[2] = 0;
     for (const CellDesc& d : cells) out[2] = std::max(out[2], d.depth);

@@ -123,6 +123,15 @@ def test_cells_take_the_place_of_other_scratch(pkg, orc):
         assert held[1] - held[0] >= 4 * 16 * m and held[1] == held[2] == held[3]
 
 
+def test_word_slots_of_short_calls(pkg):
+    """One step needs one slot per cell and slice: 46 cells, of which fewer
+    have children, on 8 slices (element by element) and the tail, 1 KB each,
+    4 for the roots, and the plan's tables."""
+    with pkg.Plan(288, 250, "int32", 1) as plan:
+        assert plan.info()["sched_transport"] == 2 and plan.info()["sched_cells"] == 46
+        assert plan.info()["scratch_bytes"] < 9 * (2 * 46 + 4) * 1024 + (1 << 17)
+
+
 def test_cells_change_of_options_and_alignment(pkg, orc):
     """One plan, calls of different kinds in a row: aligned and unaligned
     buffers (other slice counts over the same counters), other block counts,
