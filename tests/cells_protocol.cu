@@ -182,3 +182,17 @@ extern "C" int words_protocol(int p, int64_t m, int esize, int single, int b, in
     }
     return 0;
 }
+
+// The base of the next call's counters and flags of a plan on cells (walk:
+// those of the counters kernels): returned, and set where `set` is not
+// negative.  -1 after a CUDA error.
+extern "C" long long cells_base(void* plan, int walk, long long set)
+{
+    const Plan* P = static_cast<const Plan*>(plan);
+    uint32_t* const at = reinterpret_cast<uint32_t*>(walk ? P->walk.d : P->words.d) + 3;
+    uint32_t base = uint32_t(set);
+    if (cudaDeviceSynchronize() != cudaSuccess) return -1;
+    if (set >= 0 && cudaMemcpy(at, &base, sizeof base, cudaMemcpyHostToDevice) != cudaSuccess) return -1;
+    if (cudaMemcpy(&base, at, sizeof base, cudaMemcpyDeviceToHost) != cudaSuccess) return -1;
+    return base;
+}

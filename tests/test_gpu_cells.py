@@ -8,10 +8,13 @@ first cut edges (p = 15, 16, 36), ragged last levels; slices of one unit, of
 32, partly filled, several to a warp, of two blocks in a step; blocks that
 start and end inside a
 16-byte unit or lie within one, rows with a ragged tail."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
 
+import cells_util
 from gpu_util import bits, empty_like_ranks, expect_bits, host_inputs, to_device
 
 pytestmark = pytest.mark.gpu
@@ -154,6 +157,57 @@ def test_cells_change_of_options_and_alignment(pkg, orc):
             call(xs, ys)
             plan.sync()
             _check(ys, want, "step %d" % step)
+
+
+RESTART = 1 << 29  # counters and flags start from 0 again (schedule_cells.cuh, kRestart)
+
+
+@pytest.fixture(scope="module")
+def base_of(tmp_path_factory):
+    L = cells_util.load(str(tmp_path_factory.mktemp("cells")))
+    L.cells_base.restype = ctypes.c_longlong
+
+    def base(plan, walk, value=-1):
+        got = L.cells_base(ctypes.c_void_p(plan._h), int(walk), ctypes.c_longlong(value))
+        assert got >= 0
+        return got
+    return base
+
+
+@pytest.mark.parametrize("run,p,m,b", [("dual", 36, 1003, 3), ("dual", 1152, 515, 4),
+                                       ("dual", 100, 40009, 5), ("single", 255, 20003, 9),
+                                       ("reduce_bcast", 100, 40009, 5)])
+@pytest.mark.parametrize("before", [1, 40], ids=["at_once", "later"])
+def test_cells_restart_of_the_numbers(pkg, orc, base_of, run, p, m, b, before):
+    """Calls across the point where counters and flags start from 0 again.
+    Calls on unaligned buffers, which use other slots than those on aligned
+    ones, leave small numbers behind first: were they not cleared, the same
+    numbers would mean another call's values afterwards."""
+    kind, dev = "int32", torch.device("cuda:0")
+    topo = "dual" if run == "dual" else "single"
+    with pkg.Plan(p, m, kind, b, topology=topo) as plan:
+        info = plan.info()
+        assert info["sched_cells"] > 0
+        walk = run == "reduce_bcast" or info["sched_transport"] == 1
+
+        def calls(count, pad, seed):
+            v = host_inputs(kind, seed, p, m, lo=-1000, hi=1000)
+            want = expect_bits(orc.tree_fold(v, orc.I32, orc.DUAL if topo == "dual" else orc.SINGLE))
+            xs, _k = to_device(v, kind, dev, pad_front=pad)
+            for k in range(count):
+                ys, _y = empty_like_ranks(xs, pad_front=pad)
+                (plan.allreduce_reduce_bcast if run == "reduce_bcast" else plan.allreduce_schedule)(xs, ys)
+                plan.sync()
+                _check(ys, want, "seed %d call %d" % (seed, k))
+
+        calls(2, 1, 1)
+        calls(1, 0, 2)
+        assert 0 < base_of(plan, walk) < 10000
+        base_of(plan, walk, RESTART - before)
+        calls(4 + before // 2, 0, 3)
+        assert base_of(plan, walk) < 10000
+        calls(3, 1, 4)
+        calls(2, 0, 5)
 
 
 @pytest.mark.parametrize("p,m", [(30, 777), (100, 40009)], ids=["words", "counters"])
