@@ -4,7 +4,10 @@ Each case draws, from its own seeded generator, the rank count p (1 to
 3000), m, the block count b, the element type, the topology, the fused
 layout, the schedule kernel's transport, CTA layout, column slices and ranks
 per CTA, and the buffer layout (separate, in place, or only 4-byte aligned), then
-checks every output of both kernels bit for bit against the oracle's fold.
+checks every output of both kernels bit for bit against the oracle's fold; the
+schedule runs with the options drawn and with all of them automatic, which is
+on subtree cells where they fit (a single tree also runs the reduction, then
+broadcast on them).
 The draws reach combinations no hand-written case names -- blocks of two
 lengths cut into slices, ragged tails under every layout, deep trees with
 few columns -- and a mismatch names its case number, which reproduces it.
@@ -89,11 +92,16 @@ def test_random_configuration(pkg, orc, k):
         mode = c["mode"]
         if mode == 3 and plan.info()["max_depth"] < 3:
             mode = 0  # the split layout needs trees of depth >= 3
-        for run in ("fused", "schedule"):
+        automatic = ("cells", "cells_rb") if c["topology"] == "single" else ("cells",)
+        for run in ("fused", *automatic, "schedule"):
             xs, ys, _keep = _buffers(x, kind, c["layout"], dev)
             if run == "fused":
                 plan.set(pkg.OPT_FUSED_MODE, mode)
                 plan.allreduce(xs, ys)
+            elif run == "cells":
+                plan.allreduce_schedule(xs, ys)
+            elif run == "cells_rb":
+                plan.allreduce_reduce_bcast(xs, ys)
             else:
                 plan.set(pkg.OPT_SCHED_TRANSPORT, c["transport"])
                 plan.set(pkg.OPT_SCHED_LAYOUT, c["sched_layout"])
@@ -162,11 +170,13 @@ def test_random_large_configuration(pkg, orc, k):
         mode = c["mode"]
         if mode == 3 and plan.info()["max_depth"] < 3:
             mode = 0
-        for run in ("fused", "schedule"):
+        for run in ("fused", "cells", "schedule"):
             yt = torch.full_like(xt, -3)
             if run == "fused":
                 plan.set(pkg.OPT_FUSED_MODE, mode)
                 plan.allreduce(xs, list(yt.unbind(0)))
+            elif run == "cells":
+                plan.allreduce_schedule(xs, list(yt.unbind(0)))
             else:
                 plan.set(pkg.OPT_SCHED_TRANSPORT, c["transport"])
                 plan.set(pkg.OPT_SCHED_LAYOUT, c["sched_layout"])
