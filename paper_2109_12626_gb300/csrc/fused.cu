@@ -159,18 +159,21 @@ int fused_auto_mode(const Plan* P)
 }
 
 // Inputs of which L2 holds a thirtieth at most are loaded past L1 at normal L2
-// priority (FarUnit), where few or many ranks share a column (min of 3 runs,
-// two places in memory): p = 1152, m = 2^22 float32 5405 against 5427 us, m =
-// 2^20 1476 against 1491, m = 5000000 6475 against 6518; p = 4094, m = 2^19
-// 2851 against 2875; p = 32, m = 2^27 4910 against 4914 and 4916 against 4960;
-// p = 2, m = 2^29 1427 against 1434.  Between, the streaming hints are level
-// or better (p = 64, m = 3 2^24 3710 against 3714; p = 127, m = 10^7 1505
-// against 1514; p = 288, m = 2^22 1397 against 1400), and at 1 to 2 GB all are
-// level.
+// priority (FarUnit) instead of with the streaming hints.  Both measured on
+// the same buffers in turn, four places in memory, medians of 9 (streaming,
+// normal; they differ by 0.05 to 0.3 % from run to run): p = 1152 float32,
+// m = 2^22 5317 and 5272 us, int32, m = 2^20 1395 and 1369; p = 4094,
+// m = 2^19 2534 and 2498; p = 288 float32, m = 2^24 5419 and 5372; p = 128,
+// m = 2^24 2498 and 2465; p = 64, m = 2^26 4966 and 4960; p = 32, m = 2^27
+// 4926 and 4915; p = 2, m = 2^29 1459 and 1452.  At the line they are level
+// (p = 32, m = 2^25; p = 512, m = 2^21; p = 288, m = 2^22 1372 and 1376), and
+// below it the streaming hints lead where ranks are few to a walk (p = 128,
+// m = 2^22 624 and 633, m = 2^21 316 and 329; p = 288, m = 2^21 693 and 703;
+// but p = 1152, m = 3 2^18 1051 and 1039).
 constexpr int64_t kFarBytes = int64_t(4) << 30;
 static bool far_inputs(const Plan* P)
 {
-    return (P->p <= 32 || P->p >= 512) && int64_t(P->p) * P->m * P->esize >= kFarBytes;
+    return int64_t(P->p) * P->m * P->esize >= kFarBytes;
 }
 
 // On rows of 4-byte elements that are only 4-byte aligned the shared-memory

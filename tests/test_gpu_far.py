@@ -19,7 +19,7 @@ def pkg():
 LIMIT = (4 << 30) // 4
 
 
-@pytest.mark.parametrize("p,mode", [(2, 1), (7, 1), (32, 1), (32, 3), (512, 3), (1152, 3)])
+@pytest.mark.parametrize("p,mode", [(2, 1), (7, 1), (32, 1), (100, 1), (32, 3), (288, 3), (512, 3), (1152, 3)])
 @pytest.mark.parametrize("over", [False, True], ids=["below", "above"])
 @pytest.mark.parametrize("in_place", [False, True], ids=["separate", "in_place"])
 def test_far_inputs_sum(pkg, p, mode, over, in_place):
