@@ -78,7 +78,6 @@ struct Unit<Op, true> {
     __device__ __forceinline__ static T op(const T& a, const T& b) { return Op::vec(a, b); }
     __device__ __forceinline__ static void copy(uint4* slot, const char* p) { cp_async16(slot, p); }
     __device__ __forceinline__ static T ld(const char* p) { return ld_l2(p); }
-    __device__ __forceinline__ static T ld_once(const char* p) { return ld_stream(p); }
     __device__ __forceinline__ static void st_keep(char* p, const T& v) { st_l2(p, v); }
     __device__ __forceinline__ static void st(char* p, const T& v) { st_stream(p, v); }
     // the unit's words, whether all carry the flag
@@ -110,7 +109,6 @@ struct Unit<Op, false> {
         for (int w = 0; w < T::kWords; w++) cp_async4(dst + w, p + 4 * w);
     }
     __device__ __forceinline__ static T ld(const char* p) { return ld_one_l2<Op>(p); }
-    __device__ __forceinline__ static T ld_once(const char* p) { return ld_one_stream<Op>(p); }
     __device__ __forceinline__ static void st_keep(char* p, const T& v) { st_one_l2<Op>(p, v); }
     __device__ __forceinline__ static void st(char* p, const T& v) { st_one_stream<Op>(p, v); }
     __device__ __forceinline__ static bool recv(const u64* p, uint32_t flag, T& v)
