@@ -1,5 +1,7 @@
-// schedule.cu -- the schedule-faithful persistent kernel of
-// dpdr_allreduce_schedule: Algorithm 1 run by every virtual rank.
+// schedule.cu -- the schedule-faithful persistent kernel with a warp group
+// per virtual rank, on counters: dpdr_allreduce_schedule where a schedule
+// option is set or the subtree cells (schedule_cells.cuh) do not fit, and
+// dpdr_allreduce_schedule_noalloc.  Algorithm 1 run by every virtual rank.
 //
 // Rank i runs rounds j = 0..b+d_i (d_i = depth).  Each round has the three
 // bidirectional steps of Algorithm 1, in order:

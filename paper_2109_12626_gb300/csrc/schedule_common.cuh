@@ -1,6 +1,7 @@
-// schedule_common.cuh -- device pieces shared by the two transports of the
-// schedule-faithful kernel: counters and block reads (schedule.cu) and
-// flagged words (schedule_ll.cu).
+// schedule_common.cuh -- device pieces shared by the schedule kernels: with a
+// warp group per rank, on counters (schedule.cu) or flagged words
+// (schedule_ll.cu), and on subtree cells (schedule_walk.cuh,
+// schedule_words.cu).
 #pragma once
 
 #include "dpdr_internal.h"

@@ -1,5 +1,7 @@
 // schedule_ll.cu -- the low-latency transport of the schedule-faithful
-// kernel (dpdr_allreduce_schedule on short pipeline blocks).
+// kernel with a warp group per virtual rank (dpdr_allreduce_schedule on short
+// pipeline blocks where a schedule option is set or the subtree cells do not
+// fit).
 //
 // Same virtual ranks, rounds, steps and bracketing as schedule.cu
 // (Algorithm 1 for every rank i, rounds j = 0..b+d_i, the exchanges with

@@ -3,18 +3,21 @@
 // words between them (dpdr_allreduce_schedule where every schedule option is
 // automatic and the inputs are small; schedule_cells.cuh).
 //
-// The schedule is Algorithm 1's, round by round: in round j every rank takes
-// its children's partial blocks j, forms Y[j] = t1 (.) (t0 (.) x_i), hands it
-// to its parent (the dual roots exchange theirs) and receives final block
-// j - d_i, which its parent received in round j - 1.
+// The schedule is Algorithm 1's: in round j every rank takes its children's
+// partial blocks j, forms Y[j] = t1 (.) (t0 (.) x_i), hands it to its parent
+// (the dual roots exchange theirs) and receives final block j - d_i, which its
+// parent received in round j - 1.  What passes in a round is not always a
+// block of the partition, though: a warp's rounds are its column slices, up
+// to two blocks' worth of them side by side (Columns), with the blocks in
+// their order; a long block takes several rounds.
 //
 // What bounds it: the chain of exchanges from the leaves to the roots and
 // back.  One trip through L2 takes 0.3 us on one die and 0.5 us across, and
 // with one warp group per rank (schedule_ll.cu) there is one per tree level
 // each way, about 1 us each with the polling loop; a cell takes three levels
-// to one.  p = 288, m = 250 int32 in 11.7 us against 20.0 (captured calls,
-// warm), p = 1152, m = 1 in 12.4 against 20.5, m = 4096 in 26 against 71,
-// p = 36, m = 80000 in 17 against 47.
+// to one.  p = 288, m = 250 int32 in 10.7 us against 20.0 (captured calls,
+// warm), p = 1152, m = 1 in 11.8 against 20.5, m = 4096 in 22.0 against 71,
+// p = 36, m = 80000 in 14.6 against 47.
 //
 // Exchanges between cells go through slots of flagged words: every 32-bit
 // word travels with the step's flag in one 64-bit store and the receiver
@@ -70,7 +73,7 @@ struct WordsArgs {
     Columns col;
     int64_t wait_ns;
     int slots;           // word_slots
-    int ncells, root0, root1;  // cells of the roots (root0 -1: one tree)
+    int ncells, root0;   // root0: cell of the lower root (-1: one tree)
     int used;            // flag values the call uses
     int skip_rank;
 };
@@ -424,7 +427,6 @@ int schedule_words_launch(Plan* P, cudaStream_t s)
     a.wait_ns = P->wait_ns;
     a.ncells = C.n;
     a.root0 = C.root0;
-    a.root1 = C.root1;
     a.used = S.steps + 1;
     a.skip_rank = P->skip_rank;
     return cell_launch(words_kernel_for(P->dtype, vec), &a, int64_t(C.n) * lines, kWarps, 0, s);
