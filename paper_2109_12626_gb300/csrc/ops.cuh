@@ -98,7 +98,7 @@ struct MatF32 {
     }
 };
 
-__host__ __device__ __forceinline__ int64_t lmin(int64_t a, int64_t b) { return a < b ? a : b; }
+__device__ __forceinline__ int64_t lmin(int64_t a, int64_t b) { return a < b ? a : b; }
 
 // ------------------------------------------------------------ memory units
 // Streaming hints: inputs are read once (evict-first), outputs written once.

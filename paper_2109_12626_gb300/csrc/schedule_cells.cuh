@@ -183,7 +183,8 @@ __host__ __device__ __forceinline__ Extent extent(const Columns& c, const Pos& a
         }
         u += int64_t(at.g) * 32;
     }
-    return Extent{u, u < e && (tail || at.j < c.b) ? int(lmin(e - u, 32)) : 0};
+    if (u >= e || (!tail && at.j >= c.b)) return Extent{u, 0};
+    return Extent{u, e - u < 32 ? int(e - u) : 32};
 }
 // The first slice of a warp from `at` on that holds units, which `at` moves on
 // to: blocks differ by a unit, so a slice past the end of one block may have

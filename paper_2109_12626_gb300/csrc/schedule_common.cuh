@@ -52,7 +52,7 @@ __device__ __forceinline__ uint64_t now_ns()
 // blocks (q = floor(m/b), rem = m mod b: the first rem blocks are one longer).
 __host__ __device__ __forceinline__ int64_t block_start(int64_t q, int64_t rem, int j)
 {
-    return int64_t(j) * q + lmin(j, rem);
+    return int64_t(j) * q + (j < rem ? j : rem);
 }
 
 // Start of column slice g (of n) of the element range [s, e): even shares,
