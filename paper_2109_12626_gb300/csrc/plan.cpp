@@ -38,6 +38,7 @@ int cuda_fail_c(cudaError_t e, const char* what)
 
 int cuda_fail(cudaError_t e, const char* what)
 {
+    if (e == cudaErrorMemoryAllocation) cudaGetLastError();  // refused: nothing else is wrong
     std::string m = std::string(what) + ": " + cudaGetErrorString(e);
     return fail(e == cudaErrorMemoryAllocation ? DPDR_ERR_OOM : DPDR_ERR_CUDA, m);
 }
@@ -415,6 +416,21 @@ extern "C" int dpdr_plan_query(dpdr_plan_t h, int* parent, int* child0,
     return DPDR_OK;
 }
 
+// Sets an option of the schedule kernels and lays them out anew; where that
+// fails (no memory for the tables, a layout that does not fit), the plan goes
+// on as it was.
+static int set_schedule(Plan* P, int* option, int64_t v)
+{
+    const int was = *option;
+    *option = int(v);
+    const int rc = schedule_configure(P);
+    if (rc) {
+        *option = was;
+        schedule_configure(P);
+    }
+    return rc;
+}
+
 extern "C" int dpdr_plan_set(dpdr_plan_t h, int key, int64_t v)
 {
     Plan* P = reinterpret_cast<Plan*>(h);
@@ -445,49 +461,27 @@ extern "C" int dpdr_plan_set(dpdr_plan_t h, int key, int64_t v)
     case DPDR_OPT_SCHED_THREADS:
         if (v != 0 && (v < 64 || v > 256 || v % 32))
             return fail(DPDR_ERR_INVALID, "schedule threads: 0 or 64..256, multiple of 32");
-        P->sched_threads = int(v);
-        return schedule_configure(P);
+        return set_schedule(P, &P->sched_threads, v);
     case DPDR_OPT_SCHED_RANKS_PER_CTA:
         if (v < 0 || v > P->p) return fail(DPDR_ERR_INVALID, "ranks per CTA out of range");
-        P->sched_rpc = int(v);
-        return schedule_configure(P);
-    case DPDR_OPT_SCHED_LAYOUT: {
+        return set_schedule(P, &P->sched_rpc, v);
+    case DPDR_OPT_SCHED_LAYOUT:
         if (v < 0 || v > 2) return fail(DPDR_ERR_INVALID, "schedule layout: 0, 1 or 2");
-        const int was = P->sched_layout;
-        P->sched_layout = int(v);
-        const int rc = schedule_configure(P);
-        if (rc) {
-            P->sched_layout = was;
-            schedule_configure(P);
-        }
-        return rc;
-    }
+        return set_schedule(P, &P->sched_layout, v);
     case DPDR_OPT_SCHED_COPY:
         if (v < 0 || v > 2) return fail(DPDR_ERR_INVALID, "schedule copy: 0, 1 or 2");
-        P->sched_copy = int(v);
-        return schedule_configure(P);
+        return set_schedule(P, &P->sched_copy, v);
     case DPDR_OPT_SCHED_SLICES:
         if (v < 0 || v > kMaxSlices) return fail(DPDR_ERR_INVALID, "slices: 0..1024");
-        P->sched_slices = int(v);
-        return schedule_configure(P);
+        return set_schedule(P, &P->sched_slices, v);
     case DPDR_OPT_SPLIT_DEPTH: {
         if (v < -1 || v > P->max_depth) return fail(DPDR_ERR_INVALID, "split depth out of range");
         P->split_depth = int(v);
         return fused_split_prepare(P, true, P->split_depth);
     }
-    case DPDR_OPT_SCHED_TRANSPORT: {
+    case DPDR_OPT_SCHED_TRANSPORT:
         if (v < 0 || v > 2) return fail(DPDR_ERR_INVALID, "schedule transport: 0, 1 or 2");
-        const int was = P->sched_transport;
-        P->sched_transport = int(v);
-        if (schedule_transport(P) == 2) {
-            const int rc = schedule_ll_prepare(P);
-            if (rc) {
-                P->sched_transport = was;
-                return rc;
-            }
-        }
-        return schedule_configure(P);
-    }
+        return set_schedule(P, &P->sched_transport, v);
     case DPDR_OPT_HOST_PATH:
         if (v < 0 || v > 2) return fail(DPDR_ERR_INVALID, "host path: 0, 1 or 2");
         P->host_path = int(v);
@@ -506,8 +500,7 @@ extern "C" int dpdr_plan_set(dpdr_plan_t h, int key, int64_t v)
         if (ring_slot(&tmp) > P->ring_slot_bytes)
             return fail(DPDR_ERR_INVALID,
                         "fewer blocks than the plan was built for: make a new plan");
-        P->b = nb;
-        return schedule_configure(P);
+        return set_schedule(P, &P->b, nb);
     }
     default:
         return fail(DPDR_ERR_INVALID, "unknown option");

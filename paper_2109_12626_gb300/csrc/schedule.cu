@@ -1174,6 +1174,7 @@ int schedule_configure(Plan* P)
 int schedule_launch(Plan* P, cudaStream_t s, int algo)
 {
     if (P->m == 0) return DPDR_OK;
+    if (!P->d_sched) return fail(DPDR_ERR_INVALID, "schedule kernel not prepared");
     SchedArgs a;
     a.x = P->d_x;
     a.y = P->d_y;

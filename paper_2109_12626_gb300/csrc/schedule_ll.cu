@@ -385,7 +385,7 @@ int schedule_ll_prepare(Plan* P)
 int schedule_ll_launch(Plan* P, cudaStream_t s)
 {
     if (P->m == 0) return DPDR_OK;
-    if (!P->d_ll) return fail(DPDR_ERR_INVALID, "schedule words not prepared");
+    if (!P->d_ll || !P->d_sched) return fail(DPDR_ERR_INVALID, "schedule words not prepared");
     LLArgs a;
     a.x = P->d_x;
     a.y = P->d_y;

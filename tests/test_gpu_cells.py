@@ -126,6 +126,21 @@ def test_cells_take_the_place_of_other_scratch(pkg, orc):
         assert held[1] - held[0] >= 4 * 16 * m and held[1] == held[2] == held[3]
 
 
+@pytest.mark.parametrize("key,value", [("OPT_SCHED_TRANSPORT", 1), ("OPT_SCHED_TRANSPORT", 2),
+                                       ("OPT_SCHED_LAYOUT", 1), ("OPT_SCHED_THREADS", 64),
+                                       ("OPT_SCHED_COPY", 2), ("OPT_SCHED_RANKS_PER_CTA", 1)])
+def test_option_that_memory_cannot_hold(pkg, key, value):
+    """Four exchange slots of a 137 GB block, or word arrays, are more than
+    the GPU has: the option is refused and the plan stays on cells."""
+    with pkg.Plan(2, 1 << 35, "int32", 1) as plan:
+        before = plan.info()
+        assert before["sched_cells"] > 0
+        with pytest.raises(pkg.DpdrError) as e:
+            plan.set(getattr(pkg, key), value)
+        assert e.value.status == pkg.DPDR_ERR_OOM
+        assert plan.info() == before
+
+
 def test_word_slots_of_short_calls(pkg):
     """One step needs one slot per cell and slice: 46 cells, of which fewer
     have children, on 8 slices (element by element) and the tail, 1 KB each,
