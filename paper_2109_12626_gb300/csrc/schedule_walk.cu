@@ -29,8 +29,8 @@ int schedule_walk_prepare(Plan* P)
     const int tree = P->r0 >= 0 ? P->p - P->p / 2 : P->p;
     std::vector<CellDesc> desc;
     if (P->max_depth + 1 >= walk::kPast) return DPDR_OK;
-    if (!make_cells(P, tree <= walk::kRanks ? walk::kRanks : 16, walk::kLevels, kMaxWarpsPerSm * P->num_sms / 2, &C,
-                    &desc))
+    if (!make_cells(P, tree <= walk::kRanks ? walk::kRanks : 16, walk::kLevels,
+                    kMaxWarpsPerSm * P->num_sms / 2, &C, &desc))
         return DPDR_OK;
     int occ = 1 << 20;
     for (int algo = 0; algo < (P->topo == DPDR_TOPO_SINGLE ? 2 : 1); algo++)

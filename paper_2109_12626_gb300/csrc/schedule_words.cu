@@ -257,7 +257,8 @@ struct Runner {
                     send(s->up_out + (t & (a.slots - 1)) * kSlot, flag, now, v);
                 } else if (s->dual) {
                     send(s->dual_out + (t & (kDualSlots - 1)) * kSlot, flag, now, v);
-                    if (!recv<1>(&s->dual_in, (t & (kDualSlots - 1)) * kSlot, 1, flag, now, in, c.j, 2)) return;
+                    if (!recv<1>(&s->dual_in, (t & (kDualSlots - 1)) * kSlot, 1, flag, now, in, c.j, 2))
+                        return;
                     v = s->cell == a.root0 ? U::op(v, in[0]) : U::op(in[0], v);
                 }
                 c.advance(a.col);
@@ -397,7 +398,8 @@ int schedule_words_prepare(Plan* P)
     }
     C.warps = std::min(occ[0], occ[1]) * P->num_sms * kWarps;
     std::vector<CellDesc> desc;
-    if (!make_cells(P, kRanks, kLevels, C.warps / 2, &C, &desc)) return DPDR_OK;  // a slice and the tail do not fit
+    if (!make_cells(P, kRanks, kLevels, C.warps / 2, &C, &desc))
+        return DPDR_OK;  // a slice and the tail do not fit
     C.off_scratch = 256 + (sizeof(CellDesc) * desc.size() + 255) / 256 * 256;
     C.scratch = std::max(slot_words(P, cell_slices(P, C, false)), slot_words(P, cell_slices(P, C, true))) *
                 sizeof(u64);

@@ -172,8 +172,10 @@ extern "C" int words_protocol(int p, int64_t m, int esize, int single, int b, in
     std::map<std::vector<char>, bool> seen;
     for (int g = 0; g < S.n + c.tail; g++) {
         const std::vector<char> live =
-            esize == 4 ? (vec ? line_rounds<SumI32, true>(c, g, empty) : line_rounds<SumI32, false>(c, g, empty))
-                       : (vec ? line_rounds<MatU32, true>(c, g, empty) : line_rounds<MatU32, false>(c, g, empty));
+            esize == 4 ? (vec ? line_rounds<SumI32, true>(c, g, empty)
+                              : line_rounds<SumI32, false>(c, g, empty))
+                       : (vec ? line_rounds<MatU32, true>(c, g, empty)
+                              : line_rounds<MatU32, false>(c, g, empty));
         if (int(live.size()) > S.steps) return 3;  // more than the call's flags
         out[0] = std::max(out[0], int(live.size()));
         if (seen[live]) continue;
