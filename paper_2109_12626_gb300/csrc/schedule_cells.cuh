@@ -145,8 +145,9 @@ struct Columns {
 };
 
 // The lane's unit of a slice: byte offset in every row, whether it is there.
-struct Spot {
-    int64_t off;
+template <class I>
+struct SpotOf {
+    I off;
     bool on;
 };
 
@@ -162,38 +163,41 @@ struct Pos {
     }
 };
 
-// A slice's units: the first, and how many (up to 32).
+// A slice's units: the first, and how many (up to 32).  I: an integer that
+// holds every element's number.
+template <class I>
 struct Extent {
-    int64_t u;
+    I u;
     int n;
 };
 
-template <class Op, bool kVec>
-__host__ __device__ __forceinline__ Extent extent(const Columns& c, const Pos& at, bool tail)
+template <class Op, bool kVec, class I>
+__host__ __device__ __forceinline__ Extent<I> extent(const Columns& c, const Pos& at, bool tail)
 {
     constexpr int E = Unit<Op, kVec>::kElems;
-    int64_t u = sched::block_start(c.q, c.rem, at.j), e = sched::block_start(c.q, c.rem, at.j + 1);
+    const I m = I(c.m);
+    I u = sched::block_start(I(c.q), I(c.rem), at.j), e = sched::block_start(I(c.q), I(c.rem), at.j + 1);
     if (tail) {
-        u = c.m - c.m % Op::kEpv;
-        e = c.m;
+        u = m - m % Op::kEpv;
+        e = m;
     } else {
         if (E > 1) {
             u = (u + E - 1) / E;
-            e = e == c.m ? e / E : (e + E - 1) / E;
+            e = e == m ? e / E : (e + E - 1) / E;
         }
-        u += int64_t(at.g) * 32;
+        u += I(at.g) * 32;
     }
-    if (u >= e || (!tail && at.j >= c.b)) return Extent{u, 0};
-    return Extent{u, e - u < 32 ? int(e - u) : 32};
+    if (u >= e || (!tail && at.j >= c.b)) return Extent<I>{u, 0};
+    return Extent<I>{u, e - u < 32 ? int(e - u) : 32};
 }
 // The first slice of a warp from `at` on that holds units, which `at` moves on
 // to: blocks differ by a unit, so a slice past the end of one block may have
 // units in the next.  False when there is none.
-template <class Op, bool kVec>
-__host__ __device__ __forceinline__ bool next_slice(const Columns& c, Pos& at, bool tail, Extent& x)
+template <class Op, bool kVec, class I>
+__host__ __device__ __forceinline__ bool next_slice(const Columns& c, Pos& at, bool tail, Extent<I>& x)
 {
     for (; at.j < c.b; at.advance(c)) {
-        x = extent<Op, kVec>(c, at, tail);
+        x = extent<Op, kVec, I>(c, at, tail);
         if (x.n) return true;
     }
     return false;

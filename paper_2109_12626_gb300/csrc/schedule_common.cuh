@@ -50,9 +50,10 @@ __device__ __forceinline__ uint64_t now_ns()
 
 // First element of block j of Algorithm 1's partition of m elements into b
 // blocks (q = floor(m/b), rem = m mod b: the first rem blocks are one longer).
-__host__ __device__ __forceinline__ int64_t block_start(int64_t q, int64_t rem, int j)
+template <class I>
+__host__ __device__ __forceinline__ I block_start(I q, I rem, int j)
 {
-    return int64_t(j) * q + (j < rem ? j : rem);
+    return I(j) * q + (I(j) < rem ? I(j) : rem);
 }
 
 // Start of column slice g (of n) of the element range [s, e): even shares,

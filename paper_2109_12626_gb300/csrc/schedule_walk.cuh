@@ -69,6 +69,7 @@ namespace dpdr {
 namespace walk {
 
 using namespace cells;
+using Spot = SpotOf<int64_t>;
 
 constexpr int kWarps = 4;     // per CTA
 constexpr int kCtas = 6;      // per SM: 80 registers, 24 warps
@@ -138,7 +139,7 @@ struct Runner {
     // of a step noted before.
     __device__ __forceinline__ Spot note(const Pos& c, int t) const
     {
-        const Extent x = extent<Op, kVec>(a.col, c, tail);
+        const Extent<int64_t> x = extent<Op, kVec, int64_t>(a.col, c, tail);
         __syncwarp();
         if (lane == 0) {
             s->past_u[t & (kPast - 1)] = x.u;

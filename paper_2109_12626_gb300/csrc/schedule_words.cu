@@ -15,9 +15,9 @@
 // back.  One trip through L2 takes 0.3 us on one die and 0.5 us across, and
 // with one warp group per rank (schedule_ll.cu) there is one per tree level
 // each way, about 1 us each with the polling loop; a cell takes three levels
-// to one.  p = 288, m = 250 int32 in 10.7 us against 20.0 (captured calls,
-// warm), p = 1152, m = 1 in 11.8 against 20.5, m = 4096 in 22.0 against 71,
-// p = 36, m = 80000 in 14.6 against 47.
+// to one.  p = 288, m = 250 int32 in 10.5 us against 20.0 (captured calls,
+// warm), p = 1152, m = 1 in 11.9 against 20.5, m = 4096 in 21.2 against 71,
+// p = 36, m = 80000 in 14.2 against 47.
 //
 // Exchanges between cells go through slots of flagged words: every 32-bit
 // word travels with the step's flag in one 64-bit store and the receiver
@@ -52,6 +52,12 @@ namespace dpdr {
 namespace {
 
 using namespace cells;
+// Numbers of elements and bytes of a row: inputs on flagged words are at most
+// 24 MiB (schedule_transport).  With 64 bits finding the next slice was long
+// enough to hold up a step (p = 19, m = 39982, b = 175 int32 180 and 172 us,
+// p = 288, m = 768, b = 12 24.9 and 23.0).
+using Index = uint32_t;
+using Spot = SpotOf<Index>;
 
 constexpr int kRanks = kWordsRanks;
 constexpr int kLevels = kWordsLevels;
@@ -226,7 +232,7 @@ struct Runner {
     // The lane's unit of the warp's next slice, from `at` on; false past the last.
     __device__ __forceinline__ bool ahead(Pos& at, Spot& p) const
     {
-        Extent x{0, 0};
+        Extent<Index> x{0, 0};
         const bool there = next_slice<Op, kVec>(a.col, at, tail, x);
         p = Spot{(x.u + lane) * U::kBytes, lane < x.n};
         return there;

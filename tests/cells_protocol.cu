@@ -36,10 +36,10 @@ std::vector<char> line_rounds(const cells::Columns& c, int g, bool empty)
 {
     if (g == c.nslices) return {1};  // the tail
     std::vector<char> live;
-    cells::Extent x;
+    cells::Extent<uint32_t> x;
     if (empty)
         for (cells::Pos at(c, g); at.j < c.b; at.advance(c))
-            live.push_back(cells::extent<T, kVec>(c, at, false).n > 0);
+            live.push_back(cells::extent<T, kVec, uint32_t>(c, at, false).n > 0);
     else
         for (cells::Pos at(c, g); cells::next_slice<T, kVec>(c, at, false, x); at.advance(c))
             live.push_back(1);
